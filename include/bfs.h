@@ -129,10 +129,11 @@ bfs_status bfs_graph_set_bins(bfs_graph* g, int32_t t_small, int32_t t_large,
  * persistent run (bfs_run without BFS_GRAPH_LOOP or BFS_HOST_LOOP) that uses
  * none of BFS_OPT_WARP_AGGREGATE, BFS_OPT_HOT_WORDS, BFS_OPT_DIRECTION,
  * BFS_OPT_BITMAP_FRONTIER, BFS_OPT_L2_PREFETCH and BFS_OPT_TMA_STAGE (the
- * defaults) runs a build of the traversal kernel with those paths compiled
- * out, which keeps more of its state in registers (about 10 % faster at
- * scale 22); setting any of them switches to the full build.  Results are
- * the same either way.
+ * defaults) runs the default traversal kernel, which knows none of those
+ * paths; setting any of them switches to the kernel that does.  Results are
+ * the same either way.  On a graph uploaded without BFS_UPLOAD_NO_RELABEL into
+ * a context that allocates for itself, the default kernel also keeps 16 bytes
+ * per vertex (row class counts) beside the graph when the device has room.
  *   BFS_OPT_WARP_AGGREGATE   0/1: lanes of a warp that claim vertices in the
  *                            same 32-bit visited word merge their bits and
  *                            issue one atomicOr (default 0).

@@ -15,7 +15,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libbfs.so")
-SOURCES = ["bfs_kernels.cu", "bfs_kernels_lean.cu", "bfs_capi.cu", "bfs_server.cpp",
+SOURCES = ["bfs_kernels.cu", "bfs_single.cu", "bfs_capi.cu", "bfs_server.cpp",
            "bfs_static.cu", "bfs_relabel.cu", "bfs_tune.cpp", "bfs_butterfly.cu", "bfs_lrb.cu",
            "bfs_paths.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

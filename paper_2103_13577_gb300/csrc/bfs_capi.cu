@@ -15,9 +15,7 @@ namespace bfs {
 
 // kernels and launch helpers (bfs_kernels.cu)
 const void* plain_persistent_fn(int mb, bool staged = false);
-namespace lean {
-const void* plain_persistent_fn(int mb);
-}
+const void* single_persistent_fn(int mb);
 const void* plain_step_fn(int mb, bool staged = false);
 const void* batch_persistent_fn(int mb);
 const void* batch_step_fn(int mb);
@@ -32,7 +30,8 @@ cudaError_t launch_degree_bins(const int64_t* off, long long n, int t_small, int
 size_t relabel_scratch_bytes(long long n);
 cudaError_t relabel_graph(const int64_t* off, const int32_t* col, long long n, long long nnz,
                           int sms, int32_t* new2old, int32_t* old2new, int64_t* new_off,
-                          int32_t* new_col, void* scratch, cudaStream_t s);
+                          int32_t* new_col, void* scratch, uint16_t* cut, long long* bounds,
+                          cudaStream_t s);
 
 static thread_local std::string t_last_error;
 
@@ -237,6 +236,12 @@ Workspace* make_workspace(bfs_graph* g, DeviceAllocator* m, bool batched, cudaSt
     return ws;
 }
 
+// Vertices the default single-source kernel can reach are below this: in a
+// degree-ordered symmetric graph the isolated ones come last.
+static long long sweep_limit(const bfs_graph* g) {
+    return g->relabelled && g->symmetric ? std::max<long long>(g->n_nonzero, 1) : g->n;
+}
+
 static void fill_params(bfs_graph* g, Workspace* ws, TraversalParams& P) {
     std::memset(&P, 0, sizeof(P));
     P.n = g->n;
@@ -266,6 +271,13 @@ static void fill_params(bfs_graph* g, Workspace* ws, TraversalParams& P) {
     // traversal that runs neither does not maintain them
     const bool need_fb = g->dir_mode != 0 || g->bitmap_div > 0;
     for (int f = 0; f < 3; ++f) P.fb[f] = need_fb ? ws->fb[f] : nullptr;
+    // the default single-source kernel keeps no frontier bitmaps: the first
+    // one's memory holds its set of queued vertices
+    P.queued = ws->fb[0];
+    P.sweep_limit = sweep_limit(g);
+    P.cut = g->d_cut;
+    for (int c = 0; c < kCutClasses; ++c) P.cut_bound[c] = g->cut_bound[c];
+    P.dense_min = kDenseMin;
     P.nnz = g->nnz;
     P.bu_limit = g->relabelled ? g->n_nonzero : g->n;
     P.dir_mode = g->dir_mode;
@@ -305,17 +317,17 @@ static bfs_status grid_size(bfs_graph* g, const void* fn, int32_t* out, size_t s
     return BFS_OK;
 }
 
-// The persistent single-source kernel a traversal of g launches: the lean
-// build (bfs_kernels_lean.cu) whenever the run asks for none of the paths
-// compiled out of it, else the full one.  Both have the same launch bounds
-// and shared memory, and the lean one never uses more registers, so the
-// full kernel's resident grid is resident for either.
-static bool plain_is_lean(const bfs_graph* g) {
+// The persistent single-source kernel a traversal of g launches: the
+// default one (bfs_single.cu) whenever the run asks for none of the optional
+// paths, else the one of bfs_kernels.cu.  Both have the same launch bounds,
+// so the grid (the smaller of the two, set_plain_grids) is resident for
+// either.
+static bool plain_is_default(const bfs_graph* g) {
     return g->tma_stage == 0 && g->dir_mode == 0 && g->bitmap_div == 0 && g->hot_words == 0 &&
            g->use_match_any == 0 && g->l2_prefetch == 0;
 }
 static const void* persistent_plain_fn(const bfs_graph* g) {
-    return plain_is_lean(g) ? lean::plain_persistent_fn(g->min_blocks)
+    return plain_is_default(g) ? single_persistent_fn(g->min_blocks)
                             : plain_persistent_fn(g->min_blocks, g->tma_stage != 0);
 }
 
@@ -326,7 +338,14 @@ static bfs_status set_plain_grids(bfs_graph* g) {
     int32_t grid2 = 0;
     bfs_status st = grid_size(g, plain_step_fn(g->min_blocks, g->tma_stage != 0), &grid2, smem);
     if (st != BFS_OK) return st;
-    return grid_size(g, plain_persistent_fn(g->min_blocks, g->tma_stage != 0), &g->grid_plain, smem);
+    int32_t grid_opt = 0;
+    st = grid_size(g, plain_persistent_fn(g->min_blocks, g->tma_stage != 0), &grid_opt, smem);
+    if (st != BFS_OK) return st;
+    int32_t grid_def = 0;
+    st = grid_size(g, single_persistent_fn(g->min_blocks), &grid_def);
+    if (st != BFS_OK) return st;
+    g->grid_plain = std::min(grid_opt, grid_def);
+    return BFS_OK;
 }
 
 static bfs_status dev_status(int s) {
@@ -791,8 +810,18 @@ bfs_status bfs_graph_upload(bfs_context* ctx, const int64_t* row_off, const int3
             m->release(scratch);
             return cleanup(fail(BFS_ERR_NO_MEMORY, "device memory exhausted (renumbering)"));
         }
+        // The rows' class counts (16 bytes per vertex) are an addition that a
+        // traversal can do without: they are kept only where the library
+        // allocates for itself (a caller's arena keeps the sizes it always
+        // had) and the device has ample room for what comes after them.
+        const size_t cut_bytes = (size_t)n * kCutClasses * sizeof(uint16_t);
+        size_t mem_free = 0, mem_all = 0;
+        if (m->capacity() == 0 && cudaMemGetInfo(&mem_free, &mem_all) == cudaSuccess &&
+            mem_free / 16 > cut_bytes)
+            g->d_cut = static_cast<uint16_t*>(m->alloc(cut_bytes));
+        if (g->d_cut) g->graph_bytes += round_up(cut_bytes, kAlign);
         e = relabel_graph(g->d_off, g->d_col, n, nnz, ctx->sms, g->d_new2old, g->d_old2new, n_off,
-                          n_col, scratch, s);
+                          n_col, scratch, g->d_cut, g->cut_bound, s);
         if (e == cudaSuccess) e = cudaMemsetAsync(n_col + nnz, 0, 16 * 4, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         m->release(scratch);
@@ -837,6 +866,7 @@ bfs_status bfs_graph_free(bfs_graph* g) {
     m->release(g->d_col);
     m->release(g->d_new2old);
     m->release(g->d_old2new);
+    m->release(g->d_cut);
     delete g;
     return BFS_OK;
 }

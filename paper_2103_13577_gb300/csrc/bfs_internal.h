@@ -27,7 +27,9 @@ struct LevelCtl {
     unsigned int discovered;            // vertices claimed at this level (any degree)
     unsigned long long new_lanes;       // batched: (vertex, lane) pairs discovered
     unsigned long long front_lanes;     // batched: lanes with a non-empty frontier
-    unsigned long long pad[1];
+    unsigned int clear_word;            // dense level: 2^32 - 1 - first bitmap word with an
+                                        // unvisited vertex (0: none)
+    unsigned int pad;
 };
 
 struct GridBarrier {
@@ -65,6 +67,16 @@ struct BinQueue {
     int64_t chunk_cap;     // chunk-start slots
 };
 
+// Rows of a degree-ordered graph list their entries by the target's degree
+// class, heaviest first; class c holds the targets of degree >= kCutDegree[c]
+// that no lighter-numbered class holds, the rest come last.
+constexpr int kCutClasses = 8;
+constexpr int kCutDegree[kCutClasses] = {1024, 256, 128, 64, 32, 16, 8, 4};
+
+// Entries from which a level of the default single-source kernel runs dense
+// (an eighth of it where the level suits, see open_level).
+constexpr long long kDenseMin = 1ll << 23;
+
 struct TraversalParams {
     // graph (device numbering)
     int64_t n;
@@ -79,6 +91,15 @@ struct TraversalParams {
     int32_t chunk_cta;
     // workspace
     uint32_t* visited;        // plain: 1 bit per vertex
+    uint32_t* queued;         // default single-source kernel: vertices already in a frontier
+                              // (a dense level's sweep takes visited & ~queued)
+    long long dense_min;      // default single-source kernel: a level whose frontier has at
+                              // least this many entries runs dense
+    const uint16_t* cut;      // nullable, [kCutClasses][n]: entries of each row in classes 0..c
+                              // (at most 65535)
+    long long cut_bound[kCutClasses];  // vertices of degree >= kCutDegree[c]: their ids are below
+    long long sweep_limit;    // default single-source kernel: vertices a level can reach are
+                              // below this
     BinQueue q[2][kBins];
     LevelCtl* ctl;            // [3]
     GridBarrier* bar;

@@ -97,23 +97,35 @@ __global__ void rel_newdeg_kernel(const int64_t* off, const int32_t* new2old, lo
     }
 }
 
-// One warp per new row; columns renamed through old2new and each row
-// stably partitioned into three groups by the new id of the neighbour:
-// vertices of degree >= 256, of degree >= 16, and the rest (new ids are in
-// decreasing degree-bucket order, so the groups are id ranges [0, h1),
-// [h1, h2), [h2, n)).  A bottom-up level checks neighbours in row order, and
-// the heavy neighbours first are the ones most likely in the frontier.
+// Vertices of each cut class come first in the new order: bounds[c] of them
+// (key = 32 - bucket, bucket = floor(log2 deg) + 1: deg >= 2^k <=> key <= 31 - k).
+struct CutBounds {
+    long long b[kCutClasses];
+};
+__global__ void rel_bounds_kernel(const unsigned long long* key_start, long long ntiles,
+                                  CutBounds* out) {
+    if (threadIdx.x < kCutClasses) {
+        constexpr int deg[kCutClasses] = {kCutDegree[0], kCutDegree[1], kCutDegree[2], kCutDegree[3],
+                                          kCutDegree[4], kCutDegree[5], kCutDegree[6], kCutDegree[7]};
+        const int lg = 31 - __clz(deg[threadIdx.x]);
+        out->b[threadIdx.x] = (long long)key_start[(long long)(32 - lg) * ntiles];
+    }
+}
+
+// One warp per new row; columns renamed through old2new and each row stably
+// partitioned by the degree class of the neighbour, heaviest first (new ids
+// are in decreasing degree-bucket order, so the classes are id ranges).  A
+// bottom-up level checks neighbours in row order, and the heavy ones are the
+// most likely in the frontier; a top-down level that knows every vertex
+// below a class's bound to be visited skips the row's entries up to that
+// class -- cut[c][row], when asked for, says how many they are.
 __global__ void rel_columns_kernel(const int64_t* off, const int32_t* col, const int32_t* new2old,
                                    const int32_t* old2new, const int64_t* new_off, long long n,
-                                   const unsigned long long* key_start, long long ntiles,
-                                   int32_t* new_col) {
-    // key = 32 - bucket, bucket = floor(log2 deg) + 1: deg >= 256 <=> key <= 23
-#ifdef BFS_NO_ROW_PARTITION
-    const long long h1 = n, h2 = n;
-#else
-    const long long h1 = (long long)key_start[24ll * ntiles];
-    const long long h2 = (long long)key_start[28ll * ntiles];
-#endif
+                                   const CutBounds* bounds, uint16_t* cut, int32_t* new_col) {
+    constexpr int kClasses = kCutClasses + 1;
+    long long bound[kCutClasses];
+#pragma unroll
+    for (int c = 0; c < kCutClasses; ++c) bound[c] = bounds->b[c];
     const long long nwarps = (long long)gridDim.x * (blockDim.x / 32);
     const int lane = threadIdx.x & 31;
     unsigned lt;
@@ -122,27 +134,57 @@ __global__ void rel_columns_kernel(const int64_t* off, const int32_t* col, const
          i += nwarps) {
         const int32_t o = new2old[i];
         const long long b = off[o], d = off[o + 1] - b, nb = new_off[i];
-        long long c0 = 0, c1 = 0;
+        if (d == 0 && cut == nullptr) continue;
+        // lane c < kClasses counts class c, then holds where its next entry goes
+        long long mine = 0;
+        int32_t x0 = 0;
+        int g0 = -1;
         for (long long k0 = 0; k0 < d; k0 += 32) {
             const long long k = k0 + lane;
             const int32_t x = k < d ? old2new[col[b + k]] : 0;
-            c0 += __popc(__ballot_sync(0xffffffffu, k < d && x < h1));
-            c1 += __popc(__ballot_sync(0xffffffffu, k < d && x >= h1 && x < h2));
+            int g = 0;
+#pragma unroll
+            for (int c = 0; c < kCutClasses; ++c) g += x >= bound[c] ? 1 : 0;
+            if (k >= d) g = -1;
+#pragma unroll
+            for (int c = 0; c < kClasses; ++c) {
+                const unsigned m = __ballot_sync(0xffffffffu, g == c);
+                if (lane == c) mine += __popc(m);
+            }
+            x0 = x;
+            g0 = g;
         }
-        long long w0 = nb, w1 = nb + c0, w2 = nb + c0 + c1;
+        long long incl = mine;
+#pragma unroll
+        for (int s = 1; s < 16; s <<= 1) {
+            const long long y = __shfl_up_sync(0xffffffffu, incl, s);
+            if (lane >= s) incl += y;
+        }
+        if (cut && lane < kCutClasses)
+            cut[lane * n + i] = (uint16_t)(incl < 65535 ? incl : 65535);
+        long long at = nb + incl - mine;
         for (long long k0 = 0; k0 < d; k0 += 32) {
             const long long k = k0 + lane;
-            const int32_t x = k < d ? old2new[col[b + k]] : 0;
-            const int g = k >= d ? -1 : (x < h1 ? 0 : (x < h2 ? 1 : 2));
-            const unsigned m0 = __ballot_sync(0xffffffffu, g == 0);
-            const unsigned m1 = __ballot_sync(0xffffffffu, g == 1);
-            const unsigned m2 = __ballot_sync(0xffffffffu, g == 2);
-            if (g == 0) new_col[w0 + __popc(m0 & lt)] = x;
-            if (g == 1) new_col[w1 + __popc(m1 & lt)] = x;
-            if (g == 2) new_col[w2 + __popc(m2 & lt)] = x;
-            w0 += __popc(m0);
-            w1 += __popc(m1);
-            w2 += __popc(m2);
+            int32_t x = x0;
+            int g = g0;
+            if (d > 32) {   // a row of one chunk still holds its entries
+                x = k < d ? old2new[col[b + k]] : 0;
+                g = 0;
+#pragma unroll
+                for (int c = 0; c < kCutClasses; ++c) g += x >= bound[c] ? 1 : 0;
+                if (k >= d) g = -1;
+            }
+            const unsigned peers = __match_any_sync(0xffffffffu, g);
+            const long long base = __shfl_sync(0xffffffffu, at, g < 0 ? 0 : g);
+            if (g >= 0) new_col[base + __popc(peers & lt)] = x;
+            // lane c moves past its class's entries of this chunk
+            unsigned cntm = 0u;
+#pragma unroll
+            for (int c = 0; c < kClasses; ++c) {
+                const unsigned m = __ballot_sync(0xffffffffu, g == c);
+                if (lane == c) cntm = m;
+            }
+            at += __popc(cntm);
         }
     }
 }
@@ -247,10 +289,13 @@ size_t relabel_scratch_bytes(long long n) {
     return (size_t)(2 * (big + 1) * 8 + ((big + kScanBlock - 1) / kScanBlock + 2) * 8) + 1024;
 }
 
-// Builds new2old/old2new and the renumbered CSR (new_off[n+1], new_col[nnz]).
+// Builds new2old/old2new and the renumbered CSR (new_off[n+1], new_col[nnz]);
+// cut (nullable, [kCutClasses][n]) and bounds (host, [kCutClasses], written
+// when the stream has been waited for) describe the rows' degree classes.
 cudaError_t relabel_graph(const int64_t* off, const int32_t* col, long long n, long long nnz,
                           int sms, int32_t* new2old, int32_t* old2new, int64_t* new_off,
-                          int32_t* new_col, void* scratch, cudaStream_t s) {
+                          int32_t* new_col, void* scratch, uint16_t* cut, long long* bounds,
+                          cudaStream_t s) {
     const long long ntiles = (n + kRelTile - 1) / kRelTile;
     const long long table = (long long)kBuckets * ntiles;
     const long long big = table > n ? table : n;
@@ -266,11 +311,15 @@ cudaError_t relabel_graph(const int64_t* off, const int32_t* col, long long n, l
     rel_newdeg_kernel<<<sms * 4, 256, 0, s>>>(off, new2old, n, a);
     e = exclusive_scan_i64(a, n, new_off, tmp, s);
     if (e != cudaSuccess) return e;
-    rel_columns_kernel<<<sms * 8, 256, 0, s>>>(off, col, new2old, old2new, new_off, n,
-                                                reinterpret_cast<const unsigned long long*>(b), ntiles,
+    // the scan's scratch is free again: the class bounds go there
+    CutBounds* d_bounds = reinterpret_cast<CutBounds*>(a);
+    rel_bounds_kernel<<<1, 32, 0, s>>>(reinterpret_cast<const unsigned long long*>(b), ntiles, d_bounds);
+    rel_columns_kernel<<<sms * 8, 256, 0, s>>>(off, col, new2old, old2new, new_off, n, d_bounds, cut,
                                                 new_col);
     (void)nnz;
-    return cudaGetLastError();
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    return cudaMemcpyAsync(bounds, d_bounds, sizeof(CutBounds), cudaMemcpyDeviceToHost, s);
 }
 
 }  // namespace bfs

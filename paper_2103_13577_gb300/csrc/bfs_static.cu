@@ -23,9 +23,7 @@
 
 namespace bfs {
 
-namespace lean {
-const void* plain_persistent_fn(int mb);
-}
+const void* single_persistent_fn(int mb);
 
 namespace {
 
@@ -47,7 +45,7 @@ constexpr size_t kChunkCap2 = (size_t)(kStaticMaxEntries / kStaticChunkCta) + 2;
 constexpr size_t kParityBytes = a256(kQueueEntries * 4) +                                   // bin 0
                                 a256(kQueueEntries * 4) + a256(kQueueEntries * 8) + a256(kChunkCap1 * 4) +  // bin 1
                                 a256(kQueueEntries * 4) + a256(kQueueEntries * 8) + a256(kChunkCap2 * 4);   // bin 2
-constexpr size_t kStaticScratchBytes = kControlBytes + kVisitedBytes + 2 * kParityBytes;
+constexpr size_t kStaticScratchBytes = kControlBytes + 2 * kVisitedBytes + 2 * kParityBytes;
 
 }  // namespace
 }  // namespace bfs
@@ -78,7 +76,7 @@ cudaError_t setup_device(StaticDevice& d, int dev) {
     int sms = 0, nb = 0;
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, lean::plain_persistent_fn(2), kBlock, 0);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, single_persistent_fn(4), kBlock, 0);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return e;
@@ -159,7 +157,7 @@ extern "C" bfs_status bfs_run_static(const int64_t* row_off, const int32_t* col,
         return BFS_ERR_CUDA;
     }
 
-    // carve the scratch: control | visited | parity 0 queues | parity 1 queues
+    // carve the scratch: control | visited | queued | parity 0 queues | parity 1 queues
     unsigned char* p = d.scratch;
     TraversalParams P;
     std::memset(&P, 0, sizeof(P));
@@ -171,6 +169,9 @@ extern "C" bfs_status bfs_run_static(const int64_t* row_off, const int32_t* col,
     p += kControlBytes;
     P.visited = reinterpret_cast<uint32_t*>(p);
     p += kVisitedBytes;
+    P.queued = reinterpret_cast<uint32_t*>(p);
+    p += kVisitedBytes;
+    P.dense_min = kDenseMin;
     for (int par = 0; par < 2; ++par) {
         for (int b = 0; b < kBins; ++b) {
             BinQueue& Q = P.q[par][b];
@@ -188,6 +189,7 @@ extern "C" bfs_status bfs_run_static(const int64_t* row_off, const int32_t* col,
         }
     }
     P.n = n;
+    P.sweep_limit = n;
     P.nnz = nnz;
     P.bu_limit = n;
     P.off = row_off;
@@ -210,7 +212,7 @@ extern "C" bfs_status bfs_run_static(const int64_t* row_off, const int32_t* col,
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "bfs_run_static: CSR check launch");
     void* args[] = {&P};
-    e = cudaLaunchCooperativeKernel(lean::plain_persistent_fn(2), dim3(d.grid), dim3(kBlock), args, 0, s);
+    e = cudaLaunchCooperativeKernel(single_persistent_fn(4), dim3(d.grid), dim3(kBlock), args, 0, s);
     if (e != cudaSuccess) return cuda_fail(e, "bfs_run_static: cooperative launch");
     if (!stats) return BFS_OK;
     DevStats h;
