@@ -260,7 +260,10 @@ static void fill_params(bfs_graph* g, Workspace* ws, TraversalParams& P) {
     P.bar = ws->bar;
     P.stats = ws->stats;
     P.lane_vn = ws->lane_vn;
+    // frontier lane sets serve bottom-up levels, the bitmap top-down ones: one
+    // buffer is either
     P.lane_front = ws->lane_front;
+    P.full = reinterpret_cast<uint32_t*>(ws->lane_front);
     P.lane_level = ws->lane_level;
     P.timeout_ns = g->timeout_ns;
     P.debug_stall = g->debug_stall;
@@ -567,6 +570,7 @@ bfs_status run_batch_on(bfs_graph* g, Workspace* ws, const int32_t* roots, int32
     for (int level = 0;; ++level) {
         LevelCtl c;
         if ((st = read_ctl(ws, level % 3, &c, s)) != BFS_OK) return st;
+        P.level = level;
         if (ctl_empty(c)) break;
         if (P.dist_int8 && level + 1 > 126)
             return fail(BFS_ERR_DEPTH_OVERFLOW, "int8 distances: level above 126");

@@ -242,7 +242,11 @@ struct Stage {
     unsigned long long mask[kBatch ? kStageCap : 1];   // batched: new lanes of u
     int cnt;
     unsigned long long edges;                          // batched: sum deg * lanes
-    const uint32_t* hot;                               // plain: shared copy of visited[0, hot_bits)
+    const uint32_t* hot;                               // plain: shared copy of visited[0, hot_bits);
+                                                       // batched: bitmap of the vertices every live
+                                                       // lane has reached, nullptr while few have
+    const uint16_t* cut;                               // batched: entries at the front of each row
+                                                       // that lead to such vertices (nullable)
     int hot_bits;                                      // 0 when the copy is off for this level
     int disc;                                          // plain: vertices this warp claimed
     uint4* tma_buf;                  // plain, BFS_OPT_TMA_STAGE: two 1 KB staging buffers
@@ -467,6 +471,7 @@ __device__ __forceinline__ void stage_init(Stage<kBatch>& S) {
         S.cnt = 0;
         S.edges = 0ull;
         S.hot = nullptr;
+        S.cut = nullptr;
         S.hot_bits = 0;
         S.disc = 0;
         S.tma_buf = nullptr;
@@ -590,11 +595,24 @@ __device__ __forceinline__ void visit_plain_k(const TraversalParams& P, Stage<fa
 // present skip the atomic (a fire-and-forget red.or otherwise).
 // The K pairs are read in groups of kBatchProbeGroup (4 at 3 CTAs/SM: 8
 // would keep 32 registers of pairs live, which spills at that occupancy).
+// Once many vertices have been reached by every live lane, their bitmap
+// (n / 8 bytes, mostly L1 hits in degree order) is read first: it spares the
+// 16-byte read through L2 of two thirds of the entries of a scale-22
+// traversal's level 3 and of nearly all of level 4's.
 template <int K>
-__device__ __forceinline__ void visit_batch_k(const TraversalParams& P, unsigned okm,
-                                              const int32_t (&u)[K],
+__device__ __forceinline__ void visit_batch_k(const TraversalParams& P, const uint32_t* full,
+                                              unsigned okm, const int32_t (&u)[K],
                                               const uint64_t (&mask)[K]) {
     constexpr int G = K < 4 ? K : 4;
+    if (full != nullptr) {
+        uint32_t w[K];
+#pragma unroll
+        for (int j = 0; j < K; ++j) w[j] = ((okm >> j) & 1u) ? full[u[j] >> 5] : 0u;
+#pragma unroll
+        for (int j = 0; j < K; ++j)
+            if ((w[j] >> (u[j] & 31)) & 1u) okm &= ~(1u << j);
+        if (__ballot_sync(FULL_MASK, okm != 0u) == 0u) return;
+    }
 #pragma unroll
     for (int j0 = 0; j0 < K; j0 += G) {
         // visited and next of a vertex are adjacent: one 16-byte load each
@@ -618,7 +636,7 @@ template <bool kBatch, int K>
 __device__ __forceinline__ void visit_k(const TraversalParams& P, Stage<kBatch>& S, unsigned okm,
                                         const int32_t (&u)[K], const int32_t (&v)[K],
                                         const uint64_t (&mask)[K], int level, int nxt, int nslot) {
-    if constexpr (kBatch) visit_batch_k<K>(P, okm, u, mask);
+    if constexpr (kBatch) visit_batch_k<K>(P, S.hot, okm, u, mask);
     else visit_plain_k<K>(P, S, okm, u, [&](int j) { return v[j]; }, level, nxt, nslot);
 }
 
@@ -716,6 +734,11 @@ __device__ void expand_small_group(const TraversalParams& P, Stage<kBatch>& S, i
         v = __ldcg(Q.v + i);
         base = __ldg(P.off + v);
         deg = (int)(__ldg(P.off + v + 1) - base);
+        if (kBatch && S.cut) {
+            const int skip = __ldg(S.cut + v);
+            base += skip;
+            deg -= skip;
+        }
         if (kBatch) mask = __ldcg(reinterpret_cast<const unsigned long long*>(Q.mask) + i);
     }
     const int incl = warp_incl_scan(deg);
@@ -792,7 +815,8 @@ __device__ void expand_warp_range(const TraversalParams& P, Stage<kBatch>& S, co
         if (ok) {
             v = __ldcg(Q.v + ij);
             const long long base = __ldg(P.off + v), end = __ldg(P.off + v + 1);
-            const long long lo = max(eo, cs), hi = min(eo + (end - base), ce);
+            const long long skip = kBatch && S.cut ? (long long)__ldg(S.cut + v) : 0ll;
+            const long long lo = max(eo + skip, cs), hi = min(eo + (end - base), ce);
             live = hi > lo;
             a = base + (lo - eo);
             b = base + (hi - eo);
@@ -857,6 +881,7 @@ __device__ void expand_cta_chunk(const TraversalParams& P, Stage<kBatch>& S, int
     __shared__ long long s_eo[kBlock], s_base[kBlock], s_end[kBlock];
     __shared__ int32_t s_v[kBlock];
     __shared__ unsigned long long s_mask[kBatch ? kBlock : 1];
+    __shared__ uint16_t s_skip[kBatch ? kBlock : 1];
     const BinQueue& Q = P.q[cur][2];
     const int warp = threadIdx.x >> 5;
     const long long cs = item * k * (long long)P.chunk_cta;
@@ -879,6 +904,7 @@ __device__ void expand_cta_chunk(const TraversalParams& P, Stage<kBatch>& S, int
                 const long long b = base + (min(eo + (end - base), ce) - eo);
                 prefetch_cols_l2(P.col, a, min(b, a + kPrefetchAhead));
             }
+            if (kBatch) s_skip[kBatch ? threadIdx.x : 0] = S.cut ? __ldg(S.cut + v) : (uint16_t)0;
             if (kBatch)
                 s_mask[kBatch ? threadIdx.x : 0] =
                     __ldcg(reinterpret_cast<const unsigned long long*>(Q.mask) + ij);
@@ -886,7 +912,9 @@ __device__ void expand_cta_chunk(const TraversalParams& P, Stage<kBatch>& S, int
         const int nent = __syncthreads_count(ok);
         for (int k = 0; k < nent; ++k) {
             const long long eok = s_eo[k], bk = s_base[k];
-            const long long lo = max(eok, cs), hi = min(eok + (s_end[k] - bk), ce);
+            const long long lo = max(eok + (kBatch ? s_skip[kBatch ? k : 0] : 0), cs);
+            const long long hi = min(eok + (s_end[k] - bk), ce);
+            if (kBatch && hi <= lo) continue;
             expand_segment<kBatch, kStaged>(P, S, bk + (lo - eok), bk + (hi - eok), s_v[k],
                                    kBatch ? s_mask[kBatch ? k : 0] : 0ull, level, nxt, nslot,
                                    (long long)warp * 256, 256ll * kWarps);

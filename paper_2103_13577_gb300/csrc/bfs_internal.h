@@ -27,9 +27,9 @@ struct LevelCtl {
     unsigned int discovered;            // vertices claimed at this level (any degree)
     unsigned long long new_lanes;       // batched: (vertex, lane) pairs discovered
     unsigned long long front_lanes;     // batched: lanes with a non-empty frontier
-    unsigned int clear_word;            // dense level: 2^32 - 1 - first bitmap word with an
-                                        // unvisited vertex (0: none)
-    unsigned int pad;
+    unsigned int clear_word;            // 2^32 - 1 - first bitmap word with an unvisited vertex,
+                                        // batched: with one some live lane lacks (0: none)
+    unsigned int full_count;            // batched: vertices every live lane has reached
 };
 
 struct GridBarrier {
@@ -106,8 +106,9 @@ struct TraversalParams {
     DevStats* stats;
     // batched traversal state
     uint64_t* lane_vn;        // [n][2]: lanes that reached v (visited), lanes reaching v next
-    uint64_t* lane_front;     // [n]: lanes for which v is in the current frontier
-    uint8_t* lane_level;      // [n][64]: level of each lane at each vertex
+    uint64_t* lane_front;     // [n]: lanes for which v is in the current frontier (dir_mode != 0)
+    uint32_t* full;           // bitmap of the vertices every live lane has reached (dir_mode 0)
+    uint8_t* lane_level;      // [n][64 bytes]: 8 bit planes of 64 lanes' levels at each vertex
     int32_t nlanes;
     int32_t dist_int8;
     int32_t roots[64];        // caller numbering, [nlanes]

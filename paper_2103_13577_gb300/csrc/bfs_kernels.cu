@@ -342,6 +342,34 @@ __device__ void expand_bitmap_tile(const TraversalParams& P, Stage<false>& S, lo
 
 }  // inline namespace
 
+// Batched top-down levels: what the previous sweep found out about vertices
+// that every live lane has reached.  Their bitmap is used once it holds a
+// 64th of the vertices; when it holds a whole prefix of the degree order, the
+// rows skip the entries that lead there (see kCutDegree).
+__device__ __forceinline__ void batch_filters(const TraversalParams& P, Stage<true>& S,
+                                              const LevelShape& L, int level) {
+    if (lane_id() != 0) return;
+    const uint32_t* full = nullptr;
+    const uint16_t* cut = nullptr;
+    // (a level of few entries does not wait for the counters)
+    if (P.dir_mode == 0 && level > 0 && 16 * (L.edges[0] + L.edges[1] + L.edges[2]) >= P.nnz) {
+        const LevelCtl& C = P.ctl[level % 3];
+        if (64ll * __ldcg(&C.full_count) >= P.sweep_limit) {
+            full = P.full;
+            const unsigned clear = __ldcg(&C.clear_word);
+            const long long prefix = clear == 0u ? P.sweep_limit : 32ll * (0xffffffffu - clear);
+            if (P.cut != nullptr)
+                for (int c = 0; c < kCutClasses; ++c)
+                    if (P.cut_bound[c] > 0 && P.cut_bound[c] <= prefix) cut = P.cut + c * P.n;
+        }
+    }
+    S.hot = full;
+    S.cut = cut;
+}
+template <bool kBatch>
+__device__ __forceinline__ void batch_filters(const TraversalParams&, Stage<kBatch>&,
+                                              const LevelShape&, int) {}
+
 template <bool kBatch, bool kStaged = false>
 __device__ void expand_level(const TraversalParams& P, Stage<kBatch>& S, const LevelShape& L,
                              int level, uint32_t* s_hot, int dir = 0) {
@@ -368,6 +396,8 @@ __device__ void expand_level(const TraversalParams& P, Stage<kBatch>& S, const L
             S.hot = s_hot;
             S.hot_bits = words * 32;
         }
+    } else {
+        batch_filters(P, S, L, level);
     }
     __syncthreads();
     bool bottom_up = false;
@@ -637,84 +667,107 @@ __device__ void init_batch(const TraversalParams& P, long long tid, long long nt
     // distances are not filled here: emit_batch writes every (lane, vertex)
 }
 
-// Level of lane i at vertex v, one byte per lane in a vertex-major array
-// (64 bytes per vertex): a sweep's writes for one vertex stay inside its own
-// two sectors.  255 means "level >= 255, written straight into dist".
-__device__ __forceinline__ void record_lane_level(const TraversalParams& P, int lane_idx,
-                                                  long long v, int32_t cv, int level) {
-    if (level < 255) {
-        P.lane_level[v * 64 + lane_idx] = (uint8_t)level;
-    } else {
-        P.lane_level[v * 64 + lane_idx] = 255;
-        const long long idx = (long long)lane_idx * P.n + cv;
-        if (P.dist_int8) reinterpret_cast<int8_t*>(P.dist)[idx] = (int8_t)level;
-        else P.dist[idx] = level;
-    }
+// Levels per vertex and lane, bit-sliced: plane j of vertex v (a 64-bit word,
+// 8 planes or 64 bytes per vertex) holds bit j of every lane's level, so a
+// sweep gives all of a vertex's new lanes their level with one or two 16-byte
+// updates of one 32-byte sector.  Planes 4 to 7 exist from level 16 on: that
+// level's sweep clears them for the vertices reached before.  The value 255
+// means "level >= 255, written straight into dist".
+__device__ __forceinline__ ulonglong2* level_planes(const TraversalParams& P, long long v) {
+    return reinterpret_cast<ulonglong2*>(P.lane_level + v * 64);
+}
+__device__ __forceinline__ ulonglong2 plane_bits(int lvl, int pair, uint64_t lanes) {
+    return make_ulonglong2((lvl >> (2 * pair)) & 1 ? lanes : 0ull,
+                           (lvl >> (2 * pair + 1)) & 1 ? lanes : 0ull);
 }
 
-// After the last level: dist rows in the caller's numbering, one thread per
-// caller vertex (coalesced stores in every row); unreached lanes get -1.
-// Caller-order rows from the per-vertex level rows.  Four consecutive
-// caller vertices per thread: each lane row gets one 16-byte (int32) or
-// 4-byte (int8) store covering all four, when the row starts keep that
-// alignment (n a multiple of 4, dist 16-byte aligned); otherwise one store
-// per value.  A level byte of 255 marks a lane whose level (>= 255) was
-// written straight into dist: such values are left as they are.
-__device__ __forceinline__ uint32_t level_byte(const uint4& r, int b) {
-    const uint32_t w = b < 4 ? r.x : b < 8 ? r.y : b < 12 ? r.z : r.w;
-    return (w >> (8 * (b & 3))) & 0xffu;
+// Bits 4q .. 4q + 3 of x, one per byte (a 4-bit number times 2^0 + 2^7 + 2^14
+// + 2^21 puts bit i at bit 8 i, among others that the mask removes).
+__device__ __forceinline__ uint32_t spread4(uint64_t x, int q) {
+    return (((uint32_t)(x >> (4 * q)) & 0xfu) * 0x00204081u) & 0x01010101u;
+}
+// Byte b of x, sign-extended.
+template <int B>
+__device__ __forceinline__ int signed_byte(uint32_t x) {
+    int r;
+    constexpr int kSel = B | ((8 | B) << 4) | ((8 | B) << 8) | ((8 | B) << 12);
+    asm("prmt.b32 %0, %1, 0, %2;" : "=r"(r) : "r"(x), "n"(kSel));
+    return r;
 }
 
-__device__ void emit_batch(const TraversalParams& P, long long tid, long long nthreads) {
-    const bool vec = (P.n & 3) == 0 && ((uintptr_t)P.dist & 15) == 0;
-    if (vec) {
+// After the last level: dist rows in the caller's numbering, unreached lanes
+// -1, from the level planes.  `top`: no level is above it.  Four consecutive
+// caller vertices per thread: their levels of four lanes are spread to bytes,
+// transposed, and each lane row gets one 16-byte (int32) or 4-byte (int8)
+// store covering all four vertices, when the row starts keep that alignment
+// (n a multiple of 4, dist 16-byte aligned) and the levels fit 4 planes;
+// otherwise one vertex per thread and one store per value, and for levels
+// from 16 on all 8 planes, lane by lane.
+__device__ void emit_batch(const TraversalParams& P, int top, long long tid, long long nthreads) {
+    const unsigned long long* const vn = reinterpret_cast<const unsigned long long*>(P.lane_vn);
+    if ((P.n & 3) == 0 && ((uintptr_t)P.dist & 15) == 0 && top < 16) {
         const long long groups = P.n >> 2;
         for (long long g = tid; g < groups; g += nthreads) {
             const long long c0 = g << 2;
             uint64_t vis[4];
-            const uint4* lv[4];
+            ulonglong2 lo[4], hi[4];   // planes 0, 1 and 2, 3
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const long long v = P.old2new ? __ldg(P.old2new + c0 + j) : c0 + j;
-                vis[j] = __ldcg(reinterpret_cast<const unsigned long long*>(P.lane_vn) + 2 * v);
-                lv[j] = reinterpret_cast<const uint4*>(P.lane_level + v * 64);
+                vis[j] = __ldcg(vn + 2 * v);
+                lo[j] = hi[j] = make_ulonglong2(0ull, 0ull);
+                if (vis[j] != 0ull) {
+                    lo[j] = __ldcg(level_planes(P, v));
+                    hi[j] = __ldcg(level_planes(P, v) + 1);
+                }
             }
 #pragma unroll 1
-            for (int k = 0; k < 4 && 16 * k < P.nlanes; ++k) {
-                uint4 r[4];
+            for (int q = 0; 4 * q < P.nlanes; ++q) {
+                uint32_t b[4];   // of vertex j: the four lanes' levels, 0xff unreached
 #pragma unroll
                 for (int j = 0; j < 4; ++j)
-                    r[j] = vis[j] ? __ldcg(lv[j] + k) : make_uint4(0u, 0u, 0u, 0u);
+                    b[j] = (spread4(lo[j].x, q) | spread4(lo[j].y, q) << 1 | spread4(hi[j].x, q) << 2 |
+                            spread4(hi[j].y, q) << 3) |
+                           ~(spread4(vis[j], q) * 0xffu);
+                const uint32_t t0 = __byte_perm(b[0], b[1], 0x5140), t1 = __byte_perm(b[2], b[3], 0x5140);
+                const uint32_t t2 = __byte_perm(b[0], b[1], 0x7362), t3 = __byte_perm(b[2], b[3], 0x7362);
+                const uint32_t row[4] = {__byte_perm(t0, t1, 0x5410), __byte_perm(t0, t1, 0x7632),
+                                         __byte_perm(t2, t3, 0x5410), __byte_perm(t2, t3, 0x7632)};
 #pragma unroll
-                for (int b = 0; b < 16; ++b) {
-                    const int i = 16 * k + b;
-                    if (i >= P.nlanes) break;
-                    int val[4];
-                    bool deep = false;
+                for (int i = 0; i < 4; ++i) {
+                    if (4 * q + i >= P.nlanes) break;
+                    const long long idx = (long long)(4 * q + i) * P.n + c0;
+                    if (P.dist_int8)
+                        *reinterpret_cast<uint32_t*>(reinterpret_cast<int8_t*>(P.dist) + idx) = row[i];
+                    else
+                        *reinterpret_cast<int4*>(P.dist + idx) =
+                            make_int4(signed_byte<0>(row[i]), signed_byte<1>(row[i]),
+                                      signed_byte<2>(row[i]), signed_byte<3>(row[i]));
+                }
+            }
+        }
+        return;
+    }
+    if (top < 16) {
+        for (long long c = tid; c < P.n; c += nthreads) {
+            const long long v = P.old2new ? __ldg(P.old2new + c) : c;
+            const uint64_t vis = __ldcg(vn + 2 * v);
+            ulonglong2 lo = make_ulonglong2(0ull, 0ull), hi = lo;
+            if (vis != 0ull) {
+                lo = __ldcg(level_planes(P, v));
+                hi = __ldcg(level_planes(P, v) + 1);
+            }
+#pragma unroll 1
+            for (int q = 0; 4 * q < P.nlanes; ++q) {
+                uint32_t b = (spread4(lo.x, q) | spread4(lo.y, q) << 1 | spread4(hi.x, q) << 2 |
+                              spread4(hi.y, q) << 3) |
+                             ~(spread4(vis, q) * 0xffu);
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const bool hit = (vis[j] >> i) & 1ull;
-                        const int lvl = (int)level_byte(r[j], b);
-                        deep |= hit && lvl == 255;
-                        val[j] = hit ? lvl : -1;
-                    }
-                    const long long idx = (long long)i * P.n + c0;
-                    if (!deep) {
-                        if (P.dist_int8)
-                            *reinterpret_cast<uint32_t*>(reinterpret_cast<int8_t*>(P.dist) + idx) =
-                                (uint32_t)(val[0] & 0xff) | ((uint32_t)(val[1] & 0xff) << 8) |
-                                ((uint32_t)(val[2] & 0xff) << 16) | ((uint32_t)(val[3] & 0xff) << 24);
-                        else
-                            *reinterpret_cast<int4*>(P.dist + idx) =
-                                make_int4(val[0], val[1], val[2], val[3]);
-                    } else {
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            if (((vis[j] >> i) & 1ull) && val[j] == 255) continue;
-                            if (P.dist_int8) reinterpret_cast<int8_t*>(P.dist)[idx + j] = (int8_t)val[j];
-                            else P.dist[idx + j] = val[j];
-                        }
-                    }
+                for (int i = 0; i < 4; ++i, b >>= 8) {
+                    if (4 * q + i >= P.nlanes) break;
+                    const long long idx = (long long)(4 * q + i) * P.n + c;
+                    if (P.dist_int8) reinterpret_cast<int8_t*>(P.dist)[idx] = (int8_t)b;
+                    else P.dist[idx] = signed_byte<0>(b);
                 }
             }
         }
@@ -722,26 +775,25 @@ __device__ void emit_batch(const TraversalParams& P, long long tid, long long nt
     }
     for (long long c = tid; c < P.n; c += nthreads) {
         const long long v = P.old2new ? __ldg(P.old2new + c) : c;
-        const uint64_t vis = __ldcg(reinterpret_cast<const unsigned long long*>(P.lane_vn) + 2 * v);
-        const uint4* lv = reinterpret_cast<const uint4*>(P.lane_level + v * 64);
-        for (int k = 0; k < 4 && 16 * k < P.nlanes; ++k) {
-            const uint4 r = vis ? __ldcg(lv + k) : make_uint4(0u, 0u, 0u, 0u);
+        const uint64_t vis = __ldcg(vn + 2 * v);
+        ulonglong2 p[4];
 #pragma unroll
-            for (int b = 0; b < 16; ++b) {
-                const int i = 16 * k + b;
-                if (i >= P.nlanes) break;
-                const bool hit = (vis >> i) & 1ull;
-                const int lvl = (int)level_byte(r, b);
-                if (hit && lvl == 255) continue;  // deep level, already written
-                const int val = hit ? lvl : -1;
-                const long long idx = (long long)i * P.n + c;
-                if (P.dist_int8) reinterpret_cast<int8_t*>(P.dist)[idx] = (int8_t)val;
-                else P.dist[idx] = val;
-            }
+        for (int k = 0; k < 4; ++k)
+            p[k] = vis != 0ull ? __ldcg(level_planes(P, v) + k) : make_ulonglong2(0ull, 0ull);
+        for (int i = 0; i < P.nlanes; ++i) {
+            int lvl = 0;
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                lvl |= (int)((p[k].x >> i) & 1ull) << (2 * k) | (int)((p[k].y >> i) & 1ull) << (2 * k + 1);
+            const bool hit = (vis >> i) & 1ull;
+            if (hit && lvl == 255) continue;  // deep level, already written
+            const int val = hit ? lvl : -1;
+            const long long idx = (long long)i * P.n + c;
+            if (P.dist_int8) reinterpret_cast<int8_t*>(P.dist)[idx] = (int8_t)val;
+            else P.dist[idx] = val;
         }
     }
 }
-
 
 // One warp seeds all roots: duplicates share one queue entry whose mask
 // holds every lane with that root.
@@ -763,8 +815,9 @@ __device__ void seed_batch(const TraversalParams& P, Stage<true>& S) {
                 }
             }
             r = P.old2new ? __ldg(P.old2new + cr) : cr;
-            record_lane_level(P, i, r, cr, 0);
             if (first) {
+#pragma unroll
+                for (int p = 0; p < 4; ++p) level_planes(P, r)[p] = make_ulonglong2(0ull, 0ull);
                 P.lane_vn[2 * (long long)r] = mask;
                 if (P.dir_mode != 0) P.lane_front[r] = mask;
             }
@@ -784,23 +837,50 @@ __device__ void seed_batch(const TraversalParams& P, Stage<true>& S) {
 
 // Phase B of a batched level: lanes that reached v for the first time get
 // distance level + 1 and make v part of the next frontier with those lanes.
-// Byte i of the result is 0xff when bit i of m (8 bits) is set: the bits
-// are spread to one per byte by three shift-or-mask steps, then each 0x01
-// byte is multiplied up to 0xff (no carries between bytes).
-__device__ __forceinline__ unsigned long long byte_mask_of_bits(unsigned m) {
-    unsigned long long x = m & 0xffu;
-    x = (x | (x << 28)) & 0x0000000f0000000full;
-    x = (x | (x << 14)) & 0x0003000300030003ull;
-    x = (x | (x << 7)) & 0x0101010101010101ull;
-    return x * 0xffull;
+// Entries from which a batched level counts as large for its sweep.
+constexpr long long kManyEntries = 1ll << 20;
+
+// What a sweep needs to know of the level and adds up over the CTA.
+struct SweepShared {
+    int track, many;          // see open_sweep; the level expands many entries
+    uint64_t live;
+    unsigned long long full, front, pairs, edges;
+    unsigned count, clear;
+};
+
+// Thread 0, while the level's frontier is being expanded (its counters are
+// final).  Vertices that every live lane has reached are looked for (see
+// batch_filters) once the frontier holds a 64th of all (vertex, lane) pairs:
+// hardly any can be complete before, and the sweeps of small frontiers are
+// spared the ballots.  A lane without a frontier now has none later: only the
+// others count.
+__device__ __forceinline__ void open_sweep(const TraversalParams& P, SweepShared& X,
+                                           unsigned long long front_lanes,
+                                           unsigned long long pairs, bool many) {
+    X.live = front_lanes;
+    X.track = P.dir_mode == 0 &&
+              64ull * pairs >= (unsigned long long)P.sweep_limit * P.nlanes;
+    X.many = many;
+    X.full = X.front = X.pairs = X.edges = 0ull;
+    X.count = X.clear = 0u;
+}
+__device__ __forceinline__ void open_sweep(const TraversalParams& P, SweepShared& X, int level) {
+    const LevelCtl& C = P.ctl[level % 3];
+    if (threadIdx.x == 0) open_sweep(P, X, ld_cg_u64(&C.front_lanes), ld_cg_u64(&C.new_lanes), true);
+    __syncthreads();
 }
 
-__device__ void sweep_batch(const TraversalParams& P, Stage<true>& S, int level, long long tid,
-                            long long nthreads) {
+__device__ void sweep_batch(const TraversalParams& P, Stage<true>& S, SweepShared& X, int level,
+                            long long tid, long long nthreads) {
+    const uint64_t live = X.live;
+    const bool track = X.track != 0;
     const int nslot = (level + 1) % 3, nxt = (level + 1) & 1;
     const unsigned lane = lane_id();
     long long my_pairs = 0, my_full = 0;
     unsigned long long my_front = 0ull;  // lanes with a vertex in the next frontier
+    // (level 16's sweep also clears planes of vertices that got nothing new)
+    const bool skip_idle = !track && level + 1 != 16;
+    unsigned full_count = 0u, clear = 0u;
     const uint64_t all_lanes = P.nlanes >= 64 ? ~0ull : ((1ull << P.nlanes) - 1ull);
     // kSweepUnroll vertices per thread and pass, their lane-set pairs loaded
     // together; the trip count is the same for every thread (the stage push
@@ -816,13 +896,28 @@ __device__ void sweep_batch(const TraversalParams& P, Stage<true>& S, int level,
             const long long v = v0 + x * nthreads;
             vnu[x] = v < P.n ? __ldcg(pairs + v) : make_ulonglong2(0ull, 0ull);
         }
+        // most warps of a small level's sweep have nothing new: the sweep is
+        // issue-bound there, so they leave before the per-vertex work
+        uint64_t any = 0ull;
+#pragma unroll
+        for (int x = 0; x < kSweepUnroll; ++x) any |= vnu[x].y;
+        if (skip_idle && __ballot_sync(FULL_MASK, any != 0ull) == 0u) {
+            if (P.dir_mode != 0) {
+#pragma unroll
+                for (int x = 0; x < kSweepUnroll; ++x)
+                    if (v0 + x * nthreads < P.n) P.lane_front[v0 + x * nthreads] = 0ull;
+            }
+            continue;
+        }
 #pragma unroll
         for (int x = 0; x < kSweepUnroll; ++x) {
             const long long v = v0 + x * nthreads;
             uint64_t fresh = 0ull;
             bool reached_before = false;  // some lane had reached v at an earlier level
+            bool full = v >= P.sweep_limit;
             if (v < P.n) {
                 const ulonglong2 vn = vnu[x];
+                full = full || (live & ~(vn.x | vn.y)) == 0ull;
                 if (vn.y != 0ull) {
                     fresh = vn.y & ~vn.x;
                     reached_before = vn.x != 0ull;
@@ -835,26 +930,36 @@ __device__ void sweep_batch(const TraversalParams& P, Stage<true>& S, int level,
                 if (P.dir_mode != 0) P.lane_front[v] = fresh;
                 my_front |= fresh;
             }
-            // levels: one read-modify-write of the vertex's 64-byte level row
-            // (16-byte accesses, consecutive vertices' rows adjacent), bytes of
-            // the new lanes set to level + 1; bytes of lanes not reached yet are
-            // never read, so a first visit skips the read
-            if (fresh != 0ull) {
-                uint4* row = reinterpret_cast<uint4*>(P.lane_level + v * 64);
-                uint4 q[4];
-    #pragma unroll
-                for (int k = 0; k < 4; ++k)
-                    q[k] = reached_before ? __ldcg(row + k) : make_uint4(0, 0, 0, 0);
-                const int lvl = level + 1 < 255 ? level + 1 : 255;
-                const unsigned long long lvl8 = (unsigned long long)lvl * 0x0101010101010101ull;
-                unsigned long long* w = reinterpret_cast<unsigned long long*>(q);
-    #pragma unroll
-                for (int g = 0; g < 8; ++g) {
-                    const unsigned long long bm = byte_mask_of_bits((unsigned)(fresh >> (8 * g)) & 0xffu);
-                    w[g] = (w[g] & ~bm) | (lvl8 & bm);
+            if (track) {
+                const unsigned w = __ballot_sync(FULL_MASK, full);
+                if (lane == 0 && v < P.sweep_limit) {
+                    P.full[v >> 5] = w;
+                    full_count += __popc(w);
+                    if (w != FULL_MASK) clear = max(clear, 0xffffffffu - (unsigned)(v >> 5));
                 }
-    #pragma unroll
-                for (int k = 0; k < 4; ++k) row[k] = q[k];
+            }
+            if (level + 1 == 16 && v < P.n && vnu[x].x != 0ull) {
+                level_planes(P, v)[2] = make_ulonglong2(0ull, 0ull);
+                level_planes(P, v)[3] = make_ulonglong2(0ull, 0ull);
+            }
+            // the new lanes' level: a first visit writes the planes, a later one
+            // adds to those that the level's bits name
+            if (fresh != 0ull) {
+                const int lvl = level + 1 < 255 ? level + 1 : 255;
+                ulonglong2* const planes = level_planes(P, v);
+                ulonglong2 z[4];   // all reads before the first write: one round trip
+#pragma unroll
+                for (int p = 0; p < 4; ++p) {
+                    z[p] = make_ulonglong2(0ull, 0ull);
+                    if (reached_before && ((lvl >> (2 * p)) & 3) != 0) z[p] = __ldcg(planes + p);
+                }
+#pragma unroll
+                for (int p = 0; p < 4; ++p) {
+                    const ulonglong2 y = plane_bits(lvl, p, fresh);
+                    const bool write = reached_before ? ((lvl >> (2 * p)) & 3) != 0
+                                                      : p < 2 || lvl >= 16;
+                    if (write) planes[p] = make_ulonglong2(y.x | z[p].x, y.y | z[p].y);
+                }
                 if (level + 1 >= 255) {
                     // deep levels: the distance goes straight to the output
                     const int32_t cv = P.new2old ? __ldg(P.new2old + v) : (int32_t)v;
@@ -870,28 +975,53 @@ __device__ void sweep_batch(const TraversalParams& P, Stage<true>& S, int level,
         }
     }
     stage_flush<true>(P, S, level, nxt, nslot);
-    if (P.dir_mode != 0) {
-        my_full = warp_incl_scan(my_full);
-        if (lane == 31 && my_full > 0)
-            atomicAdd(reinterpret_cast<unsigned long long*>(&P.stats->full_edges),
-                      (unsigned long long)my_full);
-        const unsigned flo = __reduce_or_sync(FULL_MASK, (unsigned)my_front);
-        const unsigned fhi = __reduce_or_sync(FULL_MASK, (unsigned)(my_front >> 32));
-        const unsigned long long fr = ((unsigned long long)fhi << 32) | flo;
-        if (lane == 0 && fr != 0ull) atomicOr(&P.ctl[nslot].front_lanes, fr);
-    }
     my_pairs = warp_incl_scan(my_pairs);
-    if (lane == 31 && my_pairs > 0) {
-        atomicAdd(reinterpret_cast<unsigned long long*>(&P.ctl[nslot].new_lanes),
-                  (unsigned long long)my_pairs);
-        atomicAdd(reinterpret_cast<unsigned long long*>(&P.stats->reached),
-                  (unsigned long long)my_pairs);
+    if (P.dir_mode != 0) my_full = warp_incl_scan(my_full);
+    const unsigned flo = __reduce_or_sync(FULL_MASK, (unsigned)my_front);
+    const unsigned fhi = __reduce_or_sync(FULL_MASK, (unsigned)(my_front >> 32));
+    const unsigned long long front = ((unsigned long long)fhi << 32) | flo;
+    // Counters: they all lie in two lines, and a line takes one reduction
+    // every 2.3 ns.  After a large level every warp has some, which would cost
+    // 10 us and more: they are added up per CTA first.  After a small one few
+    // warps have any, and the extra step is not worth its round trip.
+    LevelCtl& N = P.ctl[nslot];
+    const bool many = X.many != 0;
+    unsigned long long* const pairs_to = many ? &X.pairs : &N.new_lanes;
+    unsigned long long* const full_to =
+        many ? &X.full : reinterpret_cast<unsigned long long*>(&P.stats->full_edges);
+    unsigned long long* const edges_to =
+        many ? &X.edges : reinterpret_cast<unsigned long long*>(&P.stats->edges);
+    if (lane == 31) {
+        if (my_pairs > 0) {
+            atomicAdd(pairs_to, (unsigned long long)my_pairs);
+            if (!many)
+                atomicAdd(reinterpret_cast<unsigned long long*>(&P.stats->reached),
+                          (unsigned long long)my_pairs);
+        }
+        if (my_full > 0) atomicAdd(full_to, (unsigned long long)my_full);
     }
-    if (lane == 0 && S.edges != 0ull) {
-        atomicAdd(reinterpret_cast<unsigned long long*>(&P.stats->edges), S.edges);
+    if (lane == 0) {
+        if (front != 0ull) atomicOr(many ? &X.front : &N.front_lanes, front);
+        if (full_count > 0u) atomicAdd(many ? &X.count : &N.full_count, full_count);
+        if (clear > 0u) atomicMax(many ? &X.clear : &N.clear_word, clear);
+        if (S.edges != 0ull) atomicAdd(edges_to, S.edges);
         S.edges = 0ull;
     }
-    __syncwarp();
+    if (!many) return;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        if (X.pairs > 0ull) {
+            atomicAdd(&N.new_lanes, X.pairs);
+            atomicAdd(reinterpret_cast<unsigned long long*>(&P.stats->reached), X.pairs);
+        }
+        if (X.edges > 0ull)
+            atomicAdd(reinterpret_cast<unsigned long long*>(&P.stats->edges), X.edges);
+        if (X.full > 0ull)
+            atomicAdd(reinterpret_cast<unsigned long long*>(&P.stats->full_edges), X.full);
+        if (X.front != 0ull) atomicOr(&N.front_lanes, X.front);
+        if (X.count > 0u) atomicAdd(&N.full_count, X.count);
+        if (X.clear > 0u) atomicMax(&N.clear_word, X.clear);
+    }
 }
 
 __device__ void book_batch_level(const TraversalParams& P, int level) {
@@ -904,6 +1034,7 @@ template <int MB>
 __global__ void __launch_bounds__(kBlock, MB)
 bfs_batch_persistent(const __grid_constant__ TraversalParams P) {
     __shared__ Stage<true> s_stage[kWarps];
+    __shared__ SweepShared s_sweep;
     Stage<true>& S = s_stage[threadIdx.x >> 5];
     stage_init(S);
     const long long nthreads = (long long)gridDim.x * kBlock;
@@ -918,7 +1049,13 @@ bfs_batch_persistent(const __grid_constant__ TraversalParams P) {
         if (grid_barrier(P, epoch)) {
             stamp(P, 2);
             bool prev_bu = false;
-            for (int level = 0;; ++level) {
+            int level = 0;
+            for (;; ++level) {
+                unsigned long long front_lanes = 0ull, pairs = 0ull;
+                if (threadIdx.x == 0) {   // in flight with the counters of the shape
+                    front_lanes = ld_cg_u64(&P.ctl[level % 3].front_lanes);
+                    pairs = ld_cg_u64(&P.ctl[level % 3].new_lanes);
+                }
                 const LevelShape L = read_level(P, level);
                 if (L.cnt[0] + L.cnt[1] + L.cnt[2] == 0) break;
                 if (P.dist_int8 && level + 1 > 126) {
@@ -928,11 +1065,14 @@ bfs_batch_persistent(const __grid_constant__ TraversalParams P) {
                 book_batch_level(P, level);
                 const int dir = batch_direction(P, L, prev_bu);
                 if (dir == 2 && blockIdx.x == 0 && threadIdx.x == 0) P.stats->bu_levels += 1;
+                if (threadIdx.x == 0)
+                    open_sweep(P, s_sweep, front_lanes, pairs,
+                               L.edges[0] + L.edges[1] + L.edges[2] >= kManyEntries);
                 expand_level<true>(P, S, L, level, nullptr, dir);
                 prev_bu = dir == 2;
                 if (!grid_barrier(P, epoch)) break;
                 stamp(P, 3 + 2 * level);
-                sweep_batch(P, S, level, tid, nthreads);
+                sweep_batch(P, S, s_sweep, level, tid, nthreads);
                 if (!grid_barrier(P, epoch)) break;
                 stamp(P, 4 + 2 * level);
                 if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -943,7 +1083,7 @@ bfs_batch_persistent(const __grid_constant__ TraversalParams P) {
             }
             // every sweep is complete here (the loop exits right after a barrier
             // or before any expansion of an empty level)
-            if (ld_volatile_i32(&P.stats->abort) == 0) emit_batch(P, tid, nthreads);
+            if (ld_volatile_i32(&P.stats->abort) == 0) emit_batch(P, level, tid, nthreads);
         }
     }
     kernel_exit(P);
@@ -953,6 +1093,7 @@ template <int MB>
 __global__ void __launch_bounds__(kBlock, MB)
 bfs_batch_step(const __grid_constant__ TraversalParams P) {
     __shared__ Stage<true> s_stage[kWarps];
+    __shared__ SweepShared s_sweep;
     Stage<true>& S = s_stage[threadIdx.x >> 5];
     stage_init(S);
     const long long nthreads = (long long)gridDim.x * kBlock;
@@ -967,9 +1108,11 @@ bfs_batch_step(const __grid_constant__ TraversalParams P) {
         book_batch_level(P, P.level);
         expand_level<true>(P, S, L, P.level, nullptr);
     } else if (P.phase == 3) {
-        sweep_batch(P, S, P.level, tid, nthreads);
+        open_sweep(P, s_sweep, P.level);
+        sweep_batch(P, S, s_sweep, P.level, tid, nthreads);
     } else if (P.phase == 4) {
-        emit_batch(P, tid, nthreads);
+        // the first level with an empty frontier: the host's, or the graph loop's
+        emit_batch(P, P.graph_cond ? ld_volatile_i32(&P.stats->graph_level) : P.level, tid, nthreads);
     } else if (P.phase == 7) {
         // graph-captured loop body: expansion of the device's current level
         const int level = ld_volatile_i32(&P.stats->graph_level);
@@ -983,7 +1126,9 @@ bfs_batch_step(const __grid_constant__ TraversalParams P) {
         }
         expand_level<true>(P, S, L, level, nullptr, dir);
     } else if (P.phase == 8) {
-        sweep_batch(P, S, ld_volatile_i32(&P.stats->graph_level), tid, nthreads);
+        const int level = ld_volatile_i32(&P.stats->graph_level);
+        open_sweep(P, s_sweep, level);
+        sweep_batch(P, S, s_sweep, level, tid, nthreads);
     } else if (P.phase == 9) {
         graph_advance_batch(P);
     }

@@ -69,3 +69,29 @@ def test_dense_levels_match_oracle(kind):
         assert oracle.check_bfs(off, col, int(r), got, p.cpu().numpy())["ok"]
     g.close()
     ctx.close()
+
+
+@pytest.mark.parametrize("kind", ["skewed", "arena", "caller_order", "directed"])
+@pytest.mark.parametrize("k", [64, 5])
+def test_batched_filters_match_oracle(kind, k):
+    """Entries to vertices every live lane has reached are filtered out; a
+    lane that ends at once (an isolated root) must not keep the filter off
+    nor be affected by it."""
+    off, col = graphgen.kronecker(16, 8, seed=43)
+    if kind == "directed":
+        off, col = _directed(off, col)
+    n, nnz = len(off) - 1, len(col)
+    roots = graphgen.pick_roots(off, k, seed=8)
+    roots[k // 2] = int(np.flatnonzero(np.diff(off) == 0)[3])
+    arena = torch.empty(16 * nnz + 1024 * n, dtype=torch.uint8, device="cuda") \
+        if kind == "arena" else None
+    ctx = bfs.Context(0, arena=arena)
+    g = bfs.Graph(ctx, off, col, flags=bfs.BFS_UPLOAD_NO_RELABEL if kind == "caller_order" else 0)
+    ref, _ = oracle.bfs_multi(off, col, roots)
+    for dtype in (torch.int32, torch.int8):
+        d = torch.empty((k, n), dtype=dtype, device="cuda")
+        g.run_batch(roots, d)
+        g.batch_sync()
+        assert np.array_equal(d.cpu().numpy().astype(np.int32), ref)
+    g.close()
+    ctx.close()
