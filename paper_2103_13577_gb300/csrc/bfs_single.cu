@@ -143,9 +143,10 @@ __device__ __forceinline__ void gather_entries(const int32_t* col, WarpSegments&
 
 // ------------------------------------------------------------- work items
 // Bins 1 and 2 are cut into equal runs of 2^shift entries, one per warp item
-// (bin 2 rows span many items); bin 0 into groups of 32 rows.  Thread 0 of
-// each CTA works a level's shape out once, in shared memory: done by every
-// warp, its arithmetic was a fixed cost of 1-2 us per level.
+// (bin 2 rows span many items); bin 0 into groups of 32 rows.  Warp 0 of each
+// CTA works a level's shape out once, in shared memory: done by every warp,
+// its arithmetic was a fixed cost of 2 us per level (an almost empty level of
+// a scale-22 traversal: 7.7 -> 5.2 us).
 struct RunBin {               // bins 1 and 2
     const int32_t* chunk;
     const int64_t* eoff;
@@ -266,7 +267,7 @@ __device__ __forceinline__ void open_level(const TraversalParams& P, Level& L, i
     // are not won back: 200 k vertices, 4.5 M entries: sparse 42 us, dense 56;
     // a million vertices, 6.1 M entries: 70 and 75; 18 M: 89 and 88; scale
     // 22, 67 M: 190 and 180.  With most vertices reached 13 M entries take 50
-    // and 37 us; uniform, 20 M entries: 121 and 93.
+    // and 37 us; uniform, 20 M entries: 121 and 100.
     const bool hubs = P.cut != nullptr && P.cut_bound[kHubClass] > 0;
     const bool late = 4 * (long long)reached > P.sweep_limit;
     const bool dense =
@@ -663,8 +664,7 @@ struct SweepShared {
 // the next frontier.  A CTA takes 64 bitmap words at a time, spread evenly
 // over the bitmap: in degree order the heavy vertices, whose chunk-start
 // runs are the longest, would otherwise all fall to a few CTAs (sweep of a
-// scale-22 traversal's level 2: 49 us with consecutive words, 40 spread; 25
-// with each entry placed once instead of once per bin).  A word's 32 row
+// scale-22 traversal's level 2: 49 us with consecutive words, 40 spread).  A word's 32 row
 // offsets and caller numbers are read in order.  The first word with a
 // vertex still unvisited bounds the prefix of the order that the next
 // level's rows may skip.
