@@ -15,7 +15,7 @@ namespace bfs {
 
 // kernels and launch helpers (bfs_kernels.cu)
 const void* plain_persistent_fn(int mb, bool staged = false);
-const void* single_persistent_fn(int mb);
+const void* single_persistent_fn(int mb, bool dense);
 const void* plain_step_fn(int mb, bool staged = false);
 const void* batch_persistent_fn(int mb);
 const void* batch_step_fn(int mb);
@@ -321,17 +321,20 @@ static bfs_status grid_size(bfs_graph* g, const void* fn, int32_t* out, size_t s
 }
 
 // The persistent single-source kernel a traversal of g launches: the
-// default one (bfs_single.cu) whenever the run asks for none of the optional
-// paths, else the one of bfs_kernels.cu.  Both have the same launch bounds,
-// so the grid (the smaller of the two, set_plain_grids) is resident for
-// either.
+// default one (bfs_single.cu, in the form that its entries call for) whenever
+// the run asks for none of the optional paths, else the one of bfs_kernels.cu.
+// All have the same launch bounds, so the grid (the smaller of the two,
+// set_plain_grids) is resident for either.
 static bool plain_is_default(const bfs_graph* g) {
     return g->tma_stage == 0 && g->dir_mode == 0 && g->bitmap_div == 0 && g->hot_words == 0 &&
            g->use_match_any == 0 && g->l2_prefetch == 0;
 }
+static const void* default_plain_fn(const bfs_graph* g) {
+    return single_persistent_fn(g->min_blocks, may_run_dense(g->nnz, g->d_cut != nullptr));
+}
 static const void* persistent_plain_fn(const bfs_graph* g) {
-    return plain_is_default(g) ? single_persistent_fn(g->min_blocks)
-                            : plain_persistent_fn(g->min_blocks, g->tma_stage != 0);
+    return plain_is_default(g) ? default_plain_fn(g)
+                               : plain_persistent_fn(g->min_blocks, g->tma_stage != 0);
 }
 
 // Plain-kernel grids for the graph's shared-memory setting (both the
@@ -345,7 +348,7 @@ static bfs_status set_plain_grids(bfs_graph* g) {
     st = grid_size(g, plain_persistent_fn(g->min_blocks, g->tma_stage != 0), &grid_opt, smem);
     if (st != BFS_OK) return st;
     int32_t grid_def = 0;
-    st = grid_size(g, single_persistent_fn(g->min_blocks), &grid_def);
+    st = grid_size(g, default_plain_fn(g), &grid_def);
     if (st != BFS_OK) return st;
     g->grid_plain = std::min(grid_opt, grid_def);
     return BFS_OK;

@@ -77,6 +77,16 @@ constexpr int kCutDegree[kCutClasses] = {1024, 256, 128, 64, 32, 16, 8, 4};
 // (an eighth of it where the level suits, see open_level).
 constexpr long long kDenseMin = 1ll << 23;
 
+// Whether a level of a graph of nnz entries can run dense (a level never holds
+// more entries than the graph; open_level has the rule for one level).  Where
+// none can, the form of the default kernel without that path is launched: its
+// sparse levels keep 64 registers with 112 / 148 bytes of spills and 14.2 KB of
+// shared memory per CTA where the form with both has 388 / 532 and 19.3 KB
+// (65 k vertices, 2.1 M entries: 96 us in the form with both, 77 without).
+inline bool may_run_dense(long long nnz, bool has_cut) {
+    return (has_cut ? 8 * nnz : nnz) >= kDenseMin;
+}
+
 struct TraversalParams {
     // graph (device numbering)
     int64_t n;

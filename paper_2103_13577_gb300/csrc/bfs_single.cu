@@ -242,13 +242,14 @@ __device__ __forceinline__ void refresh_prefix(const TraversalParams& P, Level& 
 
 // Warp 0: shape of the level about to be expanded, lane b working out bin b
 // (as one thread's serial code it took 3 us of every level); block 0 books it.
+template <bool kDense>
 __device__ __forceinline__ void open_level(const TraversalParams& P, Level& L, int level) {
     const int lane = (int)lane_id();
     const int slot = level % 3, cur = level & 1;
     const int b = lane < kBins ? lane : 0;
     const unsigned long long p = ld_cg_u64(&P.ctl[slot].packed[b]);
     const unsigned discovered = __ldcg(&P.ctl[slot].discovered);
-    const unsigned clear = __ldcg(&P.ctl[slot].clear_word);
+    const unsigned clear = kDense ? __ldcg(&P.ctl[slot].clear_word) : 0u;
     const BinQueue& Q = P.q[cur][b];
     // clamped so that a recorded overflow cannot turn into a bad read
     const int cnt = (int)min((long long)(p >> kCountShift), (long long)Q.cap);
@@ -270,13 +271,13 @@ __device__ __forceinline__ void open_level(const TraversalParams& P, Level& L, i
     // and 37 us; uniform, 20 M entries: 121 and 100.
     const bool hubs = P.cut != nullptr && P.cut_bound[kHubClass] > 0;
     const bool late = 4 * (long long)reached > P.sweep_limit;
-    const bool dense =
-        E >= P.dense_min || (8 * E >= P.dense_min && P.cut != nullptr && (!hubs || late));
+    const bool dense = kDense && (E >= P.dense_min ||
+                                  (8 * E >= P.dense_min && P.cut != nullptr && (!hubs || late)));
     // Dense levels: runs of 32 to 2048 entries, two to eight per warp, so that
     // the last round of the static deal leaves few warps idle, but 512
     // entries as soon as two such runs per warp can be had.
     const int run_shift = max(min(max(fit - 2, 5), 11), min(fit - 1, 9));
-    if (lane < kBins) {
+    if (kDense && lane < kBins) {
         if (lane == 0) {
             L.v0 = Q.v;
             L.cnt0 = cnt;
@@ -295,11 +296,11 @@ __device__ __forceinline__ void open_level(const TraversalParams& P, Level& L, i
         }
     }
     if (lane == 31 && !dense) L.shape = read_level(P, level);
-    const bool swept = L.dense != 0;   // the previous level's sweep looked at every word
+    const bool swept = kDense && L.dense != 0;   // the previous level's sweep looked at every word
     long long prefix = L.prefix;
     if (swept) prefix = clear == 0u ? P.sweep_limit : 32ll * (0xffffffffu - clear);
     __syncwarp();
-    set_prefix(P, L, prefix);
+    if (kDense) set_prefix(P, L, prefix);
     if (blockIdx.x == 0 && lane >= 8 && lane < 8 + (int)(sizeof(LevelCtl) / 8))
         // clear the slot that the level after next will fill
         reinterpret_cast<unsigned long long*>(P.ctl + (level + 2) % 3)[lane - 8] = 0ull;
@@ -308,10 +309,12 @@ __device__ __forceinline__ void open_level(const TraversalParams& P, Level& L, i
         L.reached = reached;
         L.edges = E;
         L.edges_seen += (unsigned long long)E;
-        L.dense = dense;
-        L.sync = dense && !swept;
-        L.look = dense && P.cut != nullptr && late && !swept;
-        L.parts = dense && hubs && P.cut_bound[kHubClass] > prefix && !late ? 2 : 1;
+        if (kDense) {
+            L.dense = dense;
+            L.sync = dense && !swept;
+            L.look = dense && P.cut != nullptr && late && !swept;
+            L.parts = dense && hubs && P.cut_bound[kHubClass] > prefix && !late ? 2 : 1;
+        }
         if (blockIdx.x == 0) {
             if (discovered > 0) P.stats->levels = level + 1;
             P.stats->reached = (long long)L.reached;
@@ -759,25 +762,57 @@ __device__ __forceinline__ void expand_root(const TraversalParams& P, Stage<fals
                               0, 256);
 }
 
-}  // namespace
-
-template <int MB>
-__global__ void __launch_bounds__(kBlock, MB)
-bfs_single_persistent(const __grid_constant__ TraversalParams P) {
-    // one level's working memory, by the way it runs
-    __shared__ union Shared {
+// One level's working memory, by the way it runs.
+template <bool kDense>
+struct LevelMemory {
+    union {
         struct {
             Stage<false> stage[kWarps];
             WarpSegments seg[kWarps];
         } expand;
         SweepShared sweep;
-        __device__ Shared() {}
-    } s;
+    };
+    __device__ LevelMemory() {}
+};
+template <>
+struct LevelMemory<false> {
+    struct {
+        Stage<false> stage[kWarps];
+    } expand;
+};
+
+// A dense level; false when a barrier was given up.
+__device__ __forceinline__ bool dense_level(const TraversalParams& P, LevelMemory<true>& s, Level& L,
+                                            int level, unsigned long long& epoch, long long tid,
+                                            long long nthreads) {
+    if (L.sync) {
+        // the levels before ran sparse: take note of what they queued
+        const long long quads = ((P.sweep_limit + 31) / 32 + 3) / 4;
+        for (long long i = tid; i < quads; i += nthreads)
+            reinterpret_cast<uint4*>(P.queued)[i] =
+                __ldcg(reinterpret_cast<const uint4*>(P.visited) + i);
+        if (!grid_barrier(P, epoch)) return false;
+    }
+    if (L.look) refresh_prefix(P, L);
+    for (int part = 0; part < L.parts; ++part) {
+        dense_part(P, s.expand.seg[threadIdx.x >> 5], L, part);
+        if (!grid_barrier(P, epoch, true)) return false;
+        if (part + 1 < L.parts) refresh_prefix(P, L);
+    }
+    sweep_level(P, s.sweep, level);
+    return true;
+}
+
+}  // namespace
+
+template <int MB, bool kDense>
+__global__ void __launch_bounds__(kBlock, MB)
+bfs_single_persistent(const __grid_constant__ TraversalParams P) {
+    __shared__ LevelMemory<kDense> s;
     __shared__ unsigned long long epoch;
     __shared__ Level L;
     __shared__ int s_disc;
     Stage<false>& S = s.expand.stage[threadIdx.x >> 5];
-    WarpSegments& W = s.expand.seg[threadIdx.x >> 5];
     const long long nthreads = (long long)gridDim.x * kBlock;
     const long long tid = (long long)blockIdx.x * kBlock + threadIdx.x;
     // a failed validation launch (same stream, so its result is visible to
@@ -815,31 +850,18 @@ bfs_single_persistent(const __grid_constant__ TraversalParams P) {
         }
         for (int level = 0;;) {
             if (level > 0) {
-                if (threadIdx.x < 32) open_level(P, L, level);
+                if (threadIdx.x < 32) open_level<kDense>(P, L, level);
                 if (threadIdx.x == 0) s_disc = 0;
                 __syncthreads();
                 if (!L.nonempty) break;
             }
             const int nslot = (level + 1) % 3, nxt = (level & 1) ^ 1;
-            if (L.dense) {
-                if (L.sync) {
-                    // the levels before ran sparse: take note of what they queued
-                    const long long quads = ((P.sweep_limit + 31) / 32 + 3) / 4;
-                    for (long long i = tid; i < quads; i += nthreads)
-                        reinterpret_cast<uint4*>(P.queued)[i] =
-                            __ldcg(reinterpret_cast<const uint4*>(P.visited) + i);
-                    if (!grid_barrier(P, epoch)) break;
-                }
-                if (L.look) refresh_prefix(P, L);
-                bool ok = true;
-                for (int part = 0; ok && part < L.parts; ++part) {
-                    dense_part(P, W, L, part);
-                    ok = grid_barrier(P, epoch, true);
-                    if (ok && part + 1 < L.parts) refresh_prefix(P, L);
-                }
-                if (!ok) break;
-                sweep_level(P, s.sweep, level);
-            } else {
+            bool dense = false;
+            if constexpr (kDense) {
+                dense = L.dense != 0;
+                if (dense && !dense_level(P, s, L, level, epoch, tid, nthreads)) break;
+            }
+            if (!dense) {
                 stage_init(S);
                 if (level == 0) expand_root(P, S, L, root);
                 else expand_top_down<false>(P, S, L.shape, level);
@@ -857,10 +879,14 @@ bfs_single_persistent(const __grid_constant__ TraversalParams P) {
     kernel_exit(P);
 }
 
-const void* single_persistent_fn(int mb) {
-    return mb >= 4 ? (const void*)bfs_single_persistent<4>
-         : mb == 3 ? (const void*)bfs_single_persistent<3>
-                   : (const void*)bfs_single_persistent<2>;
+const void* single_persistent_fn(int mb, bool dense) {
+    if (dense)
+        return mb >= 4 ? (const void*)bfs_single_persistent<4, true>
+             : mb == 3 ? (const void*)bfs_single_persistent<3, true>
+                       : (const void*)bfs_single_persistent<2, true>;
+    return mb >= 4 ? (const void*)bfs_single_persistent<4, false>
+         : mb == 3 ? (const void*)bfs_single_persistent<3, false>
+                   : (const void*)bfs_single_persistent<2, false>;
 }
 
 }  // namespace bfs

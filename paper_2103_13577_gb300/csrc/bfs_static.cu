@@ -16,6 +16,7 @@
 // at once when the check failed, so a bad index is never dereferenced.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstring>
 #include <mutex>
 
@@ -23,7 +24,7 @@
 
 namespace bfs {
 
-const void* single_persistent_fn(int mb);
+const void* single_persistent_fn(int mb, bool dense);
 
 namespace {
 
@@ -31,6 +32,20 @@ constexpr int64_t kStaticMaxVertices = 1ll << 19;   // 524,288 vertices
 constexpr int64_t kStaticMaxEntries = 1ll << 25;    // 33,554,432 adjacency entries
 constexpr int32_t kStaticTSmall = 32, kStaticTLarge = 2048;
 constexpr int32_t kStaticChunkWarp = 1024, kStaticChunkCta = 8192;
+
+// The kernel: the form without dense levels, built for 3 CTAs per SM (80
+// registers, no spills).  In the caller's vertex order, without row cuts, dense
+// levels do not pay up to the limits above (524,288 vertices, skewed, 32 M
+// entries: 227 us with them, 195 without; uniform, 31 M: 260 and 248).
+// 2 of the 3 CTAs per SM are launched up to 2^22 entries: a barrier waits for
+// every CTA's arrival, and these graphs have no work for more warps (uniform,
+// 100,003 vertices, 3.2 M entries: 127 us with 2, 136 with 3; skewed, 262,144
+// vertices, 8 M: 110 and 106; the two cross between 3.8 and 4.8 M).
+// 4 per SM at 64 registers was slower at most sizes: 62 us against 58 at 4,096
+// vertices, 162 against 139 at 100,003 uniform ones.
+inline const void* static_kernel() { return single_persistent_fn(3, false); }
+constexpr int64_t kStaticWideEntries = 1ll << 22;
+constexpr int kStaticNarrowCtas = 2;
 
 constexpr size_t a256(size_t x) { return (x + 255) & ~size_t(255); }
 constexpr size_t kCtlBytes = a256(3 * sizeof(LevelCtl));
@@ -45,7 +60,7 @@ constexpr size_t kChunkCap2 = (size_t)(kStaticMaxEntries / kStaticChunkCta) + 2;
 constexpr size_t kParityBytes = a256(kQueueEntries * 4) +                                   // bin 0
                                 a256(kQueueEntries * 4) + a256(kQueueEntries * 8) + a256(kChunkCap1 * 4) +  // bin 1
                                 a256(kQueueEntries * 4) + a256(kQueueEntries * 8) + a256(kChunkCap2 * 4);   // bin 2
-constexpr size_t kStaticScratchBytes = kControlBytes + 2 * kVisitedBytes + 2 * kParityBytes;
+constexpr size_t kStaticScratchBytes = kControlBytes + kVisitedBytes + 2 * kParityBytes;
 
 }  // namespace
 }  // namespace bfs
@@ -63,7 +78,7 @@ struct StaticDevice {
     std::mutex mu;
     bool ready = false;
     unsigned char* scratch = nullptr;   // device address of g_bfs_static_scratch
-    int grid = 0;
+    int sms = 0, per_sm = 0;            // SMs; resident CTAs of the kernel on each
 };
 constexpr int kMaxDevices = 64;
 StaticDevice g_static_dev[kMaxDevices];
@@ -76,13 +91,14 @@ cudaError_t setup_device(StaticDevice& d, int dev) {
     int sms = 0, nb = 0;
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, single_persistent_fn(4), kBlock, 0);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, static_kernel(), kBlock, 0);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return e;
     }
     d.scratch = static_cast<unsigned char*>(p);
-    d.grid = nb * sms;
+    d.sms = sms;
+    d.per_sm = nb;
     d.ready = true;
     return cudaSuccess;
 }
@@ -152,12 +168,14 @@ extern "C" bfs_status bfs_run_static(const int64_t* row_off, const int32_t* col,
     StaticDevice& d = g_static_dev[dev];
     e = setup_device(d, dev);
     if (e != cudaSuccess) return cuda_fail(e, "bfs_run_static: per-device set-up");
-    if (d.grid < 1) {
+    if (d.per_sm < 1) {
         set_error("bfs_run_static: traversal kernel cannot be resident");
         return BFS_ERR_CUDA;
     }
 
-    // carve the scratch: control | visited | queued | parity 0 queues | parity 1 queues
+    const int grid = d.sms * (nnz <= kStaticWideEntries ? std::min(d.per_sm, kStaticNarrowCtas) : d.per_sm);
+
+    // carve the scratch: control | visited | parity 0 queues | parity 1 queues
     unsigned char* p = d.scratch;
     TraversalParams P;
     std::memset(&P, 0, sizeof(P));
@@ -169,9 +187,6 @@ extern "C" bfs_status bfs_run_static(const int64_t* row_off, const int32_t* col,
     p += kControlBytes;
     P.visited = reinterpret_cast<uint32_t*>(p);
     p += kVisitedBytes;
-    P.queued = reinterpret_cast<uint32_t*>(p);
-    p += kVisitedBytes;
-    P.dense_min = kDenseMin;
     for (int par = 0; par < 2; ++par) {
         for (int b = 0; b < kBins; ++b) {
             BinQueue& Q = P.q[par][b];
@@ -189,7 +204,6 @@ extern "C" bfs_status bfs_run_static(const int64_t* row_off, const int32_t* col,
         }
     }
     P.n = n;
-    P.sweep_limit = n;
     P.nnz = nnz;
     P.bu_limit = n;
     P.off = row_off;
@@ -208,11 +222,11 @@ extern "C" bfs_status bfs_run_static(const int64_t* row_off, const int32_t* col,
     // the traversal kernel clears the bitmap
     e = cudaMemsetAsync(d.scratch, 0, kControlBytes, s);
     if (e != cudaSuccess) return cuda_fail(e, "bfs_run_static: clearing the control block");
-    static_csr_check<<<d.grid, kBlock, 0, s>>>(row_off, nnz > 0 ? col : nullptr, n, nnz, check);
+    static_csr_check<<<grid, kBlock, 0, s>>>(row_off, nnz > 0 ? col : nullptr, n, nnz, check);
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "bfs_run_static: CSR check launch");
     void* args[] = {&P};
-    e = cudaLaunchCooperativeKernel(single_persistent_fn(4), dim3(d.grid), dim3(kBlock), args, 0, s);
+    e = cudaLaunchCooperativeKernel(static_kernel(), dim3(grid), dim3(kBlock), args, 0, s);
     if (e != cudaSuccess) return cuda_fail(e, "bfs_run_static: cooperative launch");
     if (!stats) return BFS_OK;
     DevStats h;
