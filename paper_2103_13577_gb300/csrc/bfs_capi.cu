@@ -30,7 +30,7 @@ cudaError_t launch_degree_bins(const int64_t* off, long long n, int t_small, int
 size_t relabel_scratch_bytes(long long n);
 cudaError_t relabel_graph(const int64_t* off, const int32_t* col, long long n, long long nnz,
                           int sms, int32_t* new2old, int32_t* old2new, int64_t* new_off,
-                          int32_t* new_col, void* scratch, uint16_t* cut, long long* bounds,
+                          int32_t* new_col, void* scratch, uint16_t* cut, CutBounds* bounds,
                           cudaStream_t s);
 
 static thread_local std::string t_last_error;
@@ -236,10 +236,11 @@ Workspace* make_workspace(bfs_graph* g, DeviceAllocator* m, bool batched, cudaSt
     return ws;
 }
 
-// Vertices the default single-source kernel can reach are below this: in a
-// degree-ordered symmetric graph the isolated ones come last.
+// Vertices that a traversal can reach are below this (its root aside): in a
+// degree-ordered graph the targets without rows of their own come last, and
+// the renumbering has seen the largest target.
 static long long sweep_limit(const bfs_graph* g) {
-    return g->relabelled && g->symmetric ? std::max<long long>(g->n_nonzero, 1) : g->n;
+    return g->relabelled ? std::max<long long>(g->bounds.reach, 1) : g->n;
 }
 
 static void fill_params(bfs_graph* g, Workspace* ws, TraversalParams& P) {
@@ -279,7 +280,7 @@ static void fill_params(bfs_graph* g, Workspace* ws, TraversalParams& P) {
     P.queued = ws->fb[0];
     P.sweep_limit = sweep_limit(g);
     P.cut = g->d_cut;
-    for (int c = 0; c < kCutClasses; ++c) P.cut_bound[c] = g->cut_bound[c];
+    for (int c = 0; c < kCutClasses; ++c) P.cut_bound[c] = g->bounds.below[c];
     P.dense_min = kDenseMin;
     P.nnz = g->nnz;
     P.bu_limit = g->relabelled ? g->n_nonzero : g->n;
@@ -828,7 +829,7 @@ bfs_status bfs_graph_upload(bfs_context* ctx, const int64_t* row_off, const int3
             g->d_cut = static_cast<uint16_t*>(m->alloc(cut_bytes));
         if (g->d_cut) g->graph_bytes += round_up(cut_bytes, kAlign);
         e = relabel_graph(g->d_off, g->d_col, n, nnz, ctx->sms, g->d_new2old, g->d_old2new, n_off,
-                          n_col, scratch, g->d_cut, g->cut_bound, s);
+                          n_col, scratch, g->d_cut, &g->bounds, s);
         if (e == cudaSuccess) e = cudaMemsetAsync(n_col + nnz, 0, 16 * 4, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         m->release(scratch);

@@ -72,6 +72,10 @@ struct BinQueue {
 // that no lighter-numbered class holds, the rest come last.
 constexpr int kCutClasses = 8;
 constexpr int kCutDegree[kCutClasses] = {1024, 256, 128, 64, 32, 16, 8, 4};
+struct CutBounds {
+    long long below[kCutClasses];   // ids of the vertices of degree >= kCutDegree[c] are below
+    long long reach;                // ids of the vertices that some row leads to are below
+};
 
 // Entries from which a level of the default single-source kernel runs dense
 // (an eighth of it where the level suits, see open_level).
@@ -108,8 +112,8 @@ struct TraversalParams {
     const uint16_t* cut;      // nullable, [kCutClasses][n]: entries of each row in classes 0..c
                               // (at most 65535)
     long long cut_bound[kCutClasses];  // vertices of degree >= kCutDegree[c]: their ids are below
-    long long sweep_limit;    // default single-source kernel: vertices a level can reach are
-                              // below this
+    long long sweep_limit;    // vertices that some row leads to are below this (the default
+                              // single-source kernel's sweeps, the batched full bitmap)
     BinQueue q[2][kBins];
     LevelCtl* ctl;            // [3]
     GridBarrier* bar;

@@ -97,19 +97,18 @@ __global__ void rel_newdeg_kernel(const int64_t* off, const int32_t* new2old, lo
     }
 }
 
-// Vertices of each cut class come first in the new order: bounds[c] of them
+// Vertices of each cut class come first in the new order: below[c] of them
 // (key = 32 - bucket, bucket = floor(log2 deg) + 1: deg >= 2^k <=> key <= 31 - k).
-struct CutBounds {
-    long long b[kCutClasses];
-};
+// `reach` starts at none; rel_columns_kernel raises it.
 __global__ void rel_bounds_kernel(const unsigned long long* key_start, long long ntiles,
                                   CutBounds* out) {
     if (threadIdx.x < kCutClasses) {
         constexpr int deg[kCutClasses] = {kCutDegree[0], kCutDegree[1], kCutDegree[2], kCutDegree[3],
                                           kCutDegree[4], kCutDegree[5], kCutDegree[6], kCutDegree[7]};
         const int lg = 31 - __clz(deg[threadIdx.x]);
-        out->b[threadIdx.x] = (long long)key_start[(long long)(32 - lg) * ntiles];
+        out->below[threadIdx.x] = (long long)key_start[(long long)(32 - lg) * ntiles];
     }
+    if (threadIdx.x == 0) out->reach = 0;
 }
 
 // One warp per new row; columns renamed through old2new and each row stably
@@ -118,14 +117,16 @@ __global__ void rel_bounds_kernel(const unsigned long long* key_start, long long
 // bottom-up level checks neighbours in row order, and the heavy ones are the
 // most likely in the frontier; a top-down level that knows every vertex
 // below a class's bound to be visited skips the row's entries up to that
-// class -- cut[c][row], when asked for, says how many they are.
+// class -- cut[c][row], when asked for, says how many they are.  The largest
+// target of all rows bounds the vertices that a traversal can reach.
 __global__ void rel_columns_kernel(const int64_t* off, const int32_t* col, const int32_t* new2old,
                                    const int32_t* old2new, const int64_t* new_off, long long n,
-                                   const CutBounds* bounds, uint16_t* cut, int32_t* new_col) {
+                                   CutBounds* bounds, uint16_t* cut, int32_t* new_col) {
     constexpr int kClasses = kCutClasses + 1;
     long long bound[kCutClasses];
 #pragma unroll
-    for (int c = 0; c < kCutClasses; ++c) bound[c] = bounds->b[c];
+    for (int c = 0; c < kCutClasses; ++c) bound[c] = bounds->below[c];
+    int reach = 0;
     const long long nwarps = (long long)gridDim.x * (blockDim.x / 32);
     const int lane = threadIdx.x & 31;
     unsigned lt;
@@ -146,6 +147,7 @@ __global__ void rel_columns_kernel(const int64_t* off, const int32_t* col, const
 #pragma unroll
             for (int c = 0; c < kCutClasses; ++c) g += x >= bound[c] ? 1 : 0;
             if (k >= d) g = -1;
+            else reach = max(reach, x + 1);
 #pragma unroll
             for (int c = 0; c < kClasses; ++c) {
                 const unsigned m = __ballot_sync(0xffffffffu, g == c);
@@ -187,6 +189,8 @@ __global__ void rel_columns_kernel(const int64_t* off, const int32_t* col, const
             at += __popc(cntm);
         }
     }
+    reach = __reduce_max_sync(0xffffffffu, reach);
+    if (lane == 0 && reach > 0) atomicMax(&bounds->reach, (long long)reach);
 }
 
 // ---------------------------------------------------- exclusive scan (int64)
@@ -290,11 +294,11 @@ size_t relabel_scratch_bytes(long long n) {
 }
 
 // Builds new2old/old2new and the renumbered CSR (new_off[n+1], new_col[nnz]);
-// cut (nullable, [kCutClasses][n]) and bounds (host, [kCutClasses], written
-// when the stream has been waited for) describe the rows' degree classes.
+// cut (nullable, [kCutClasses][n]) and bounds (host, written when the stream
+// has been waited for) describe the rows' degree classes.
 cudaError_t relabel_graph(const int64_t* off, const int32_t* col, long long n, long long nnz,
                           int sms, int32_t* new2old, int32_t* old2new, int64_t* new_off,
-                          int32_t* new_col, void* scratch, uint16_t* cut, long long* bounds,
+                          int32_t* new_col, void* scratch, uint16_t* cut, CutBounds* bounds,
                           cudaStream_t s) {
     const long long ntiles = (n + kRelTile - 1) / kRelTile;
     const long long table = (long long)kBuckets * ntiles;

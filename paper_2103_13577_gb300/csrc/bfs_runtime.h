@@ -83,7 +83,7 @@ struct bfs_graph {
     int32_t* d_old2new = nullptr;     // caller numbering -> device numbering
     bool relabelled = false;
     uint16_t* d_cut = nullptr;        // [kCutClasses][n] row class counts (nullptr: not kept)
-    long long cut_bound[bfs::kCutClasses] = {};
+    bfs::CutBounds bounds = {};       // of the degree order (relabelled graphs)
     int32_t t_small = 16, t_large = 4096, chunk_warp = 128, chunk_cta = 1024;
     uint64_t bin_count[bfs::kBins] = {0, 0, 0};
     uint64_t bin_edges[bfs::kBins] = {0, 0, 0};
