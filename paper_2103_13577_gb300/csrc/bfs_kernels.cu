@@ -683,7 +683,8 @@ __device__ __forceinline__ ulonglong2 plane_bits(int lvl, int pair, uint64_t lan
 
 // Bits 4q .. 4q + 3 of x, one per byte (a 4-bit number times 2^0 + 2^7 + 2^14
 // + 2^21 puts bit i at bit 8 i, among others that the mask removes).
-__device__ __forceinline__ uint32_t spread4(uint64_t x, int q) {
+template <typename T>
+__device__ __forceinline__ uint32_t spread4(T x, int q) {
     return (((uint32_t)(x >> (4 * q)) & 0xfu) * 0x00204081u) & 0x01010101u;
 }
 // Byte b of x, sign-extended.
@@ -695,17 +696,86 @@ __device__ __forceinline__ int signed_byte(uint32_t x) {
     return r;
 }
 
+// Bytes of four vertices (byte i: lane i) to rows of four vertices: row[i]
+// byte j is b[j] byte i.
+__device__ __forceinline__ void transpose4(const uint32_t (&b)[4], uint32_t (&row)[4]) {
+    const uint32_t t0 = __byte_perm(b[0], b[1], 0x5140), t1 = __byte_perm(b[2], b[3], 0x5140);
+    const uint32_t t2 = __byte_perm(b[0], b[1], 0x7362), t3 = __byte_perm(b[2], b[3], 0x7362);
+    row[0] = __byte_perm(t0, t1, 0x5410);
+    row[1] = __byte_perm(t0, t1, 0x7632);
+    row[2] = __byte_perm(t2, t3, 0x5410);
+    row[3] = __byte_perm(t2, t3, 0x7632);
+}
+
+// Low byte of x as a level, 255 as -1.
+__device__ __forceinline__ int level_or_none(uint32_t x) { return (int)((x + 1u) & 0xffu) - 1; }
+
+// emit_batch for levels 16 to 254 and rows that allow wide stores: all 8
+// planes, 16 lanes at a time (those of four vertices and 64 lanes would take
+// 64 registers; a vertex's 64 bytes come from L1 after the first 16 lanes).
+// A million vertices, 64 lanes, 22 levels: 790 us with one store per value, 765
+// so (int8 rows 789 and 743).
+__device__ void emit_deep_rows(const TraversalParams& P, long long tid, long long nthreads) {
+    const unsigned long long* const vn = reinterpret_cast<const unsigned long long*>(P.lane_vn);
+    const long long groups = P.n >> 2;
+    for (long long g = tid; g < groups; g += nthreads) {
+        const long long c0 = g << 2;
+#pragma unroll 1
+        for (int part = 0; 16 * part < P.nlanes; ++part) {
+            uint32_t vis[4], pl[4][4];   // pl: planes 2k (low half) and 2k + 1
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const long long v = P.old2new ? __ldg(P.old2new + c0 + j) : c0 + j;
+                vis[j] = reinterpret_cast<const uint16_t*>(vn + 2 * v)[part];
+                const uint16_t* const row = reinterpret_cast<const uint16_t*>(level_planes(P, v)) + part;
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    pl[j][k] = vis[j] != 0u ? (uint32_t)row[8 * k] | (uint32_t)row[8 * k + 4] << 16 : 0u;
+            }
+#pragma unroll 1
+            for (int q = 0; q < 4 && 16 * part + 4 * q < P.nlanes; ++q) {
+                uint32_t b[4], row[4];   // levels, 0xff (no level here) where unreached
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    b[j] = ~(spread4(vis[j], q) * 0xffu);
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        b[j] |= spread4(pl[j][k], q) << (2 * k) | spread4(pl[j][k], q + 4) << (2 * k + 1);
+                }
+                transpose4(b, row);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int lane_idx = 16 * part + 4 * q + i;
+                    if (lane_idx >= P.nlanes) break;
+                    const long long idx = (long long)lane_idx * P.n + c0;
+                    if (P.dist_int8)
+                        *reinterpret_cast<uint32_t*>(reinterpret_cast<int8_t*>(P.dist) + idx) = row[i];
+                    else
+                        *reinterpret_cast<int4*>(P.dist + idx) =
+                            make_int4(level_or_none(row[i]), level_or_none(row[i] >> 8),
+                                      level_or_none(row[i] >> 16), level_or_none(row[i] >> 24));
+                }
+            }
+        }
+    }
+}
+
 // After the last level: dist rows in the caller's numbering, unreached lanes
 // -1, from the level planes.  `top`: no level is above it.  Four consecutive
 // caller vertices per thread: their levels of four lanes are spread to bytes,
 // transposed, and each lane row gets one 16-byte (int32) or 4-byte (int8)
 // store covering all four vertices, when the row starts keep that alignment
-// (n a multiple of 4, dist 16-byte aligned) and the levels fit 4 planes;
+// (n a multiple of 4, dist 16-byte aligned) and no level is above 254;
 // otherwise one vertex per thread and one store per value, and for levels
 // from 16 on all 8 planes, lane by lane.
 __device__ void emit_batch(const TraversalParams& P, int top, long long tid, long long nthreads) {
     const unsigned long long* const vn = reinterpret_cast<const unsigned long long*>(P.lane_vn);
-    if ((P.n & 3) == 0 && ((uintptr_t)P.dist & 15) == 0 && top < 16) {
+    const bool wide = (P.n & 3) == 0 && ((uintptr_t)P.dist & 15) == 0;
+    if (wide && top >= 16 && top < 255) {
+        emit_deep_rows(P, tid, nthreads);
+        return;
+    }
+    if (wide && top < 16) {
         const long long groups = P.n >> 2;
         for (long long g = tid; g < groups; g += nthreads) {
             const long long c0 = g << 2;
@@ -729,10 +799,8 @@ __device__ void emit_batch(const TraversalParams& P, int top, long long tid, lon
                     b[j] = (spread4(lo[j].x, q) | spread4(lo[j].y, q) << 1 | spread4(hi[j].x, q) << 2 |
                             spread4(hi[j].y, q) << 3) |
                            ~(spread4(vis[j], q) * 0xffu);
-                const uint32_t t0 = __byte_perm(b[0], b[1], 0x5140), t1 = __byte_perm(b[2], b[3], 0x5140);
-                const uint32_t t2 = __byte_perm(b[0], b[1], 0x7362), t3 = __byte_perm(b[2], b[3], 0x7362);
-                const uint32_t row[4] = {__byte_perm(t0, t1, 0x5410), __byte_perm(t0, t1, 0x7632),
-                                         __byte_perm(t2, t3, 0x5410), __byte_perm(t2, t3, 0x7632)};
+                uint32_t row[4];
+                transpose4(b, row);
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     if (4 * q + i >= P.nlanes) break;
