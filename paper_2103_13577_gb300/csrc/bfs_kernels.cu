@@ -713,15 +713,19 @@ __device__ __forceinline__ int level_or_none(uint32_t x) { return (int)((x + 1u)
 // emit_batch for levels 16 to 254 and rows that allow wide stores: all 8
 // planes, 16 lanes at a time (those of four vertices and 64 lanes would take
 // 64 registers; a vertex's 64 bytes come from L1 after the first 16 lanes).
-// A million vertices, 64 lanes, 22 levels: 790 us with one store per value, 765
-// so (int8 rows 789 and 743).
+// Where there are fewer groups of four vertices than threads, each 16 lanes of
+// a group are a thread of their own.  A million vertices, 64 lanes, 22 levels:
+// 790 us with one store per value, 765 so (int8 rows 789 and 743).
 __device__ void emit_deep_rows(const TraversalParams& P, long long tid, long long nthreads) {
     const unsigned long long* const vn = reinterpret_cast<const unsigned long long*>(P.lane_vn);
-    const long long groups = P.n >> 2;
-    for (long long g = tid; g < groups; g += nthreads) {
-        const long long c0 = g << 2;
+    const unsigned groups = (unsigned)(P.n >> 2), parts = (unsigned)(P.nlanes + 15) / 16;
+    const bool spread = groups < nthreads;
+    const unsigned items = spread ? groups * parts : groups;   // fewer than 2^30
+    for (unsigned it = (unsigned)tid; it < items; it += (unsigned)nthreads) {
+        const unsigned p0 = spread ? it / groups : 0u, p1 = spread ? p0 + 1u : parts;
+        const long long c0 = 4ll * (it - (spread ? p0 * groups : 0u));
 #pragma unroll 1
-        for (int part = 0; 16 * part < P.nlanes; ++part) {
+        for (unsigned part = p0; part < p1; ++part) {
             uint32_t vis[4], pl[4][4];   // pl: planes 2k (low half) and 2k + 1
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
@@ -733,7 +737,7 @@ __device__ void emit_deep_rows(const TraversalParams& P, long long tid, long lon
                     pl[j][k] = vis[j] != 0u ? (uint32_t)row[8 * k] | (uint32_t)row[8 * k + 4] << 16 : 0u;
             }
 #pragma unroll 1
-            for (int q = 0; q < 4 && 16 * part + 4 * q < P.nlanes; ++q) {
+            for (int q = 0; q < 4 && 16 * (int)part + 4 * q < P.nlanes; ++q) {
                 uint32_t b[4], row[4];   // levels, 0xff (no level here) where unreached
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
@@ -745,7 +749,7 @@ __device__ void emit_deep_rows(const TraversalParams& P, long long tid, long lon
                 transpose4(b, row);
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
-                    const int lane_idx = 16 * part + 4 * q + i;
+                    const int lane_idx = 16 * (int)part + 4 * q + i;
                     if (lane_idx >= P.nlanes) break;
                     const long long idx = (long long)lane_idx * P.n + c0;
                     if (P.dist_int8)
@@ -766,8 +770,7 @@ __device__ void emit_deep_rows(const TraversalParams& P, long long tid, long lon
 // transposed, and each lane row gets one 16-byte (int32) or 4-byte (int8)
 // store covering all four vertices, when the row starts keep that alignment
 // (n a multiple of 4, dist 16-byte aligned) and no level is above 254;
-// otherwise one vertex per thread and one store per value, and for levels
-// from 16 on all 8 planes, lane by lane.
+// otherwise one vertex per thread and one store per value.
 __device__ void emit_batch(const TraversalParams& P, int top, long long tid, long long nthreads) {
     const unsigned long long* const vn = reinterpret_cast<const unsigned long long*>(P.lane_vn);
     const bool wide = (P.n & 3) == 0 && ((uintptr_t)P.dist & 15) == 0;
@@ -848,17 +851,22 @@ __device__ void emit_batch(const TraversalParams& P, int top, long long tid, lon
 #pragma unroll
         for (int k = 0; k < 4; ++k)
             p[k] = vis != 0ull ? __ldcg(level_planes(P, v) + k) : make_ulonglong2(0ull, 0ull);
-        for (int i = 0; i < P.nlanes; ++i) {
-            int lvl = 0;
+#pragma unroll 1
+        for (int q = 0; 4 * q < P.nlanes; ++q) {
+            uint32_t b = 0u, hit = spread4(vis, q);   // four lanes' levels, and which are reached
 #pragma unroll
             for (int k = 0; k < 4; ++k)
-                lvl |= (int)((p[k].x >> i) & 1ull) << (2 * k) | (int)((p[k].y >> i) & 1ull) << (2 * k + 1);
-            const bool hit = (vis >> i) & 1ull;
-            if (hit && lvl == 255) continue;  // deep level, already written
-            const int val = hit ? lvl : -1;
-            const long long idx = (long long)i * P.n + c;
-            if (P.dist_int8) reinterpret_cast<int8_t*>(P.dist)[idx] = (int8_t)val;
-            else P.dist[idx] = val;
+                b |= spread4(p[k].x, q) << (2 * k) | spread4(p[k].y, q) << (2 * k + 1);
+#pragma unroll
+            for (int i = 0; i < 4; ++i, b >>= 8, hit >>= 8) {
+                if (4 * q + i >= P.nlanes) break;
+                const int lvl = (int)(b & 0xffu);
+                if ((hit & 1u) && lvl == 255) continue;  // deep level, already written
+                const int val = hit & 1u ? lvl : -1;
+                const long long idx = (long long)(4 * q + i) * P.n + c;
+                if (P.dist_int8) reinterpret_cast<int8_t*>(P.dist)[idx] = (int8_t)val;
+                else P.dist[idx] = val;
+            }
         }
     }
 }
