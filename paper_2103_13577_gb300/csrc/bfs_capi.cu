@@ -264,7 +264,8 @@ static void fill_params(bfs_graph* g, Workspace* ws, TraversalParams& P) {
     // frontier lane sets serve bottom-up levels, the bitmap top-down ones: one
     // buffer is either
     P.lane_front = ws->lane_front;
-    P.full = reinterpret_cast<uint32_t*>(ws->lane_front);
+    if (g->dir_mode == 0 && g->nnz >= kFilterMin)
+        P.full = reinterpret_cast<uint32_t*>(ws->lane_front);
     P.lane_level = ws->lane_level;
     P.timeout_ns = g->timeout_ns;
     P.debug_stall = g->debug_stall;

@@ -81,6 +81,13 @@ struct CutBounds {
 // (an eighth of it where the level suits, see open_level).
 constexpr long long kDenseMin = 1ll << 23;
 
+// Entries from which a batched top-down run looks for vertices that every live
+// lane has reached.  A graph of fewer gives a warp a few hundred entries per
+// level at most, and the counters cost its levels more than the entries spared
+// (64 lanes, 50 k vertices, 0.8 M entries: 154 us with them, 146 without; 131 k,
+// 2 M: 186 either way, and 600 k, 9 M: 386 with them against 411).
+constexpr long long kFilterMin = 1ll << 20;
+
 // Whether a level of a graph of nnz entries can run dense (a level never holds
 // more entries than the graph; open_level has the rule for one level).  Where
 // none can, the form of the default kernel without that path is launched: its
@@ -121,7 +128,8 @@ struct TraversalParams {
     // batched traversal state
     uint64_t* lane_vn;        // [n][2]: lanes that reached v (visited), lanes reaching v next
     uint64_t* lane_front;     // [n]: lanes for which v is in the current frontier (dir_mode != 0)
-    uint32_t* full;           // bitmap of the vertices every live lane has reached (dir_mode 0)
+    uint32_t* full;           // bitmap of the vertices every live lane has reached (nullptr:
+                              // not looked for; else the buffer of lane_front)
     uint8_t* lane_level;      // [n][64 bytes]: 8 bit planes of 64 lanes' levels at each vertex
     int32_t nlanes;
     int32_t dist_int8;

@@ -352,7 +352,7 @@ __device__ __forceinline__ void batch_filters(const TraversalParams& P, Stage<tr
     const uint32_t* full = nullptr;
     const uint16_t* cut = nullptr;
     // (a level of few entries does not wait for the counters)
-    if (P.dir_mode == 0 && level > 0 && 16 * (L.edges[0] + L.edges[1] + L.edges[2]) >= P.nnz) {
+    if (P.full != nullptr && level > 0 && 16 * (L.edges[0] + L.edges[1] + L.edges[2]) >= P.nnz) {
         const LevelCtl& C = P.ctl[level % 3];
         if (64ll * __ldcg(&C.full_count) >= P.sweep_limit) {
             full = P.full;
@@ -911,53 +911,89 @@ __device__ void seed_batch(const TraversalParams& P, Stage<true>& S) {
     __syncwarp();
 }
 
-// Phase B of a batched level: lanes that reached v for the first time get
-// distance level + 1 and make v part of the next frontier with those lanes.
 // Entries from which a batched level counts as large for its sweep.
 constexpr long long kManyEntries = 1ll << 20;
 
 // What a sweep needs to know of the level and adds up over the CTA.
 struct SweepShared {
     int track, many;          // see open_sweep; the level expands many entries
+    int publish;              // the next level needs to know which lanes have a frontier
+    int plain;                // none of these
     uint64_t live;
     unsigned long long full, front, pairs, edges;
     unsigned count, clear;
 };
+
+__device__ __forceinline__ uint64_t lanes_of(const TraversalParams& P) {
+    return P.nlanes >= 64 ? ~0ull : ((1ull << P.nlanes) - 1ull);
+}
 
 // Thread 0, while the level's frontier is being expanded (its counters are
 // final).  Vertices that every live lane has reached are looked for (see
 // batch_filters) once the frontier holds a 64th of all (vertex, lane) pairs:
 // hardly any can be complete before, and the sweeps of small frontiers are
 // spared the ballots.  A lane without a frontier now has none later: only the
-// others count.
+// others count.  Which lanes those are is asked for (two warp reductions and
+// one atomic per warp that found something) when the entries per frontier
+// vertex would bring the next frontier to that size; where it was not, every
+// lane counts as live.
 __device__ __forceinline__ void open_sweep(const TraversalParams& P, SweepShared& X,
                                            unsigned long long front_lanes,
-                                           unsigned long long pairs, bool many) {
-    X.live = front_lanes;
-    X.track = P.dir_mode == 0 &&
-              64ull * pairs >= (unsigned long long)P.sweep_limit * P.nlanes;
+                                           unsigned long long pairs, long long vertices,
+                                           long long entries, bool many) {
+    X.track = 0;
+    X.publish = P.dir_mode != 0;
+    X.live = front_lanes != 0ull ? front_lanes : lanes_of(P);
+    if (P.full != nullptr) {
+        const float all = (float)P.sweep_limit * (float)P.nlanes;
+        const float now = 64.f * (float)max(pairs, (unsigned long long)P.nlanes);
+        X.track = now >= all;
+        X.publish = now * (float)entries >= all * (float)vertices;
+    }
     X.many = many;
+    X.plain = !X.track && !many && (P.dir_mode != 0 || !X.publish);
     X.full = X.front = X.pairs = X.edges = 0ull;
     X.count = X.clear = 0u;
 }
+// The same in a launch of its own (host- and graph-driven loops).
 __device__ __forceinline__ void open_sweep(const TraversalParams& P, SweepShared& X, int level) {
-    const LevelCtl& C = P.ctl[level % 3];
-    if (threadIdx.x == 0) open_sweep(P, X, ld_cg_u64(&C.front_lanes), ld_cg_u64(&C.new_lanes), true);
+    if (threadIdx.x == 0) {
+        const LevelCtl& C = P.ctl[level % 3];
+        long long vertices = 0, entries = 0;
+#pragma unroll
+        for (int b = 0; b < kBins; ++b) {
+            const unsigned long long p = ld_cg_u64(&C.packed[b]);
+            vertices += (long long)(p >> kCountShift);
+            entries += (long long)(p & kEdgeMask);
+        }
+        open_sweep(P, X, ld_cg_u64(&C.front_lanes), ld_cg_u64(&C.new_lanes), vertices, entries,
+                   entries >= kManyEntries);
+    }
     __syncthreads();
 }
 
-__device__ void sweep_batch(const TraversalParams& P, Stage<true>& S, SweepShared& X, int level,
-                            long long tid, long long nthreads) {
-    const uint64_t live = X.live;
-    const bool track = X.track != 0;
+// Phase B of a batched level: lanes that reached v for the first time get
+// distance level + 1 and make v part of the next frontier with those lanes.
+// Two forms: kPlain for levels that need none of tracking, publishing in a
+// top-down run, counters per CTA and the clearing at level 16.  A small level's
+// sweep is a few microseconds of mostly idle warps, and the code of those it
+// would run through costs it 0.5 us (116 sweeps of a 60 x 60 mesh, 64 lanes:
+// 718 us in one form, 645 in its own).
+template <bool kPlain>
+__device__ void sweep_batch_form(const TraversalParams& P, Stage<true>& S, SweepShared& X, int level,
+                                 long long tid, long long nthreads) {
+    const uint64_t live = kPlain ? 0ull : X.live;
+    const bool track = !kPlain && X.track != 0;
+    const bool publish = kPlain ? P.dir_mode != 0 : X.publish != 0;
+    const bool clear_high = !kPlain && level + 1 == 16;
     const int nslot = (level + 1) % 3, nxt = (level + 1) & 1;
     const unsigned lane = lane_id();
     long long my_pairs = 0, my_full = 0;
     unsigned long long my_front = 0ull;  // lanes with a vertex in the next frontier
     // (level 16's sweep also clears planes of vertices that got nothing new)
-    const bool skip_idle = !track && level + 1 != 16;
+    const bool skip_idle = !track && !clear_high;
     unsigned full_count = 0u, clear = 0u;
-    const uint64_t all_lanes = P.nlanes >= 64 ? ~0ull : ((1ull << P.nlanes) - 1ull);
+    const uint64_t all_lanes = lanes_of(P);
     // kSweepUnroll vertices per thread and pass, their lane-set pairs loaded
     // together; the trip count is the same for every thread (the stage push
     // is warp-collective)
@@ -1014,7 +1050,7 @@ __device__ void sweep_batch(const TraversalParams& P, Stage<true>& S, SweepShare
                     if (w != FULL_MASK) clear = max(clear, 0xffffffffu - (unsigned)(v >> 5));
                 }
             }
-            if (level + 1 == 16 && v < P.n && vnu[x].x != 0ull) {
+            if (clear_high && v < P.n && vnu[x].x != 0ull) {
                 level_planes(P, v)[2] = make_ulonglong2(0ull, 0ull);
                 level_planes(P, v)[3] = make_ulonglong2(0ull, 0ull);
             }
@@ -1053,51 +1089,67 @@ __device__ void sweep_batch(const TraversalParams& P, Stage<true>& S, SweepShare
     stage_flush<true>(P, S, level, nxt, nslot);
     my_pairs = warp_incl_scan(my_pairs);
     if (P.dir_mode != 0) my_full = warp_incl_scan(my_full);
-    const unsigned flo = __reduce_or_sync(FULL_MASK, (unsigned)my_front);
-    const unsigned fhi = __reduce_or_sync(FULL_MASK, (unsigned)(my_front >> 32));
-    const unsigned long long front = ((unsigned long long)fhi << 32) | flo;
-    // Counters: they all lie in two lines, and a line takes one reduction
-    // every 2.3 ns.  After a large level every warp has some, which would cost
-    // 10 us and more: they are added up per CTA first.  After a small one few
-    // warps have any, and the extra step is not worth its round trip.
+    unsigned long long front = 0ull;
+    if (publish) {
+        const unsigned flo = __reduce_or_sync(FULL_MASK, (unsigned)my_front);
+        const unsigned fhi = __reduce_or_sync(FULL_MASK, (unsigned)(my_front >> 32));
+        front = ((unsigned long long)fhi << 32) | flo;
+    }
     LevelCtl& N = P.ctl[nslot];
-    const bool many = X.many != 0;
-    unsigned long long* const pairs_to = many ? &X.pairs : &N.new_lanes;
-    unsigned long long* const full_to =
-        many ? &X.full : reinterpret_cast<unsigned long long*>(&P.stats->full_edges);
-    unsigned long long* const edges_to =
-        many ? &X.edges : reinterpret_cast<unsigned long long*>(&P.stats->edges);
-    if (lane == 31) {
-        if (my_pairs > 0) {
-            atomicAdd(pairs_to, (unsigned long long)my_pairs);
-            if (!many)
-                atomicAdd(reinterpret_cast<unsigned long long*>(&P.stats->reached),
-                          (unsigned long long)my_pairs);
+    unsigned long long* const reached = reinterpret_cast<unsigned long long*>(&P.stats->reached);
+    unsigned long long* const edges = reinterpret_cast<unsigned long long*>(&P.stats->edges);
+    unsigned long long* const full_edges = reinterpret_cast<unsigned long long*>(&P.stats->full_edges);
+    if (kPlain || !X.many) {
+        if (lane == 31) {
+            if (my_pairs > 0) {
+                atomicAdd(&N.new_lanes, (unsigned long long)my_pairs);
+                atomicAdd(reached, (unsigned long long)my_pairs);
+            }
+            if (my_full > 0) atomicAdd(full_edges, (unsigned long long)my_full);
         }
-        if (my_full > 0) atomicAdd(full_to, (unsigned long long)my_full);
+        if (lane == 0) {
+            if (front != 0ull) atomicOr(&N.front_lanes, front);
+            if (full_count > 0u) atomicAdd(&N.full_count, full_count);
+            if (clear > 0u) atomicMax(&N.clear_word, clear);
+            if (S.edges != 0ull) atomicAdd(edges, S.edges);
+            S.edges = 0ull;
+        }
+        __syncwarp();
+        return;
+    }
+    // The counters all lie in two lines, and a line takes one reduction every
+    // 2.3 ns.  After a large level every warp has some, which would cost 10 us
+    // and more: they are added up per CTA first.  On smaller levels the extra
+    // step's round trip costs more than it saves.
+    if (lane == 31) {
+        if (my_pairs > 0) atomicAdd(&X.pairs, (unsigned long long)my_pairs);
+        if (my_full > 0) atomicAdd(&X.full, (unsigned long long)my_full);
     }
     if (lane == 0) {
-        if (front != 0ull) atomicOr(many ? &X.front : &N.front_lanes, front);
-        if (full_count > 0u) atomicAdd(many ? &X.count : &N.full_count, full_count);
-        if (clear > 0u) atomicMax(many ? &X.clear : &N.clear_word, clear);
-        if (S.edges != 0ull) atomicAdd(edges_to, S.edges);
+        if (front != 0ull) atomicOr(&X.front, front);
+        if (full_count > 0u) atomicAdd(&X.count, full_count);
+        if (clear > 0u) atomicMax(&X.clear, clear);
+        if (S.edges != 0ull) atomicAdd(&X.edges, S.edges);
         S.edges = 0ull;
     }
-    if (!many) return;
     __syncthreads();
     if (threadIdx.x == 0) {
         if (X.pairs > 0ull) {
             atomicAdd(&N.new_lanes, X.pairs);
-            atomicAdd(reinterpret_cast<unsigned long long*>(&P.stats->reached), X.pairs);
+            atomicAdd(reached, X.pairs);
         }
-        if (X.edges > 0ull)
-            atomicAdd(reinterpret_cast<unsigned long long*>(&P.stats->edges), X.edges);
-        if (X.full > 0ull)
-            atomicAdd(reinterpret_cast<unsigned long long*>(&P.stats->full_edges), X.full);
+        if (X.edges > 0ull) atomicAdd(edges, X.edges);
+        if (X.full > 0ull) atomicAdd(full_edges, X.full);
         if (X.front != 0ull) atomicOr(&N.front_lanes, X.front);
         if (X.count > 0u) atomicAdd(&N.full_count, X.count);
         if (X.clear > 0u) atomicMax(&N.clear_word, X.clear);
     }
+}
+
+__device__ __forceinline__ void sweep_batch(const TraversalParams& P, Stage<true>& S, SweepShared& X,
+                                            int level, long long tid, long long nthreads) {
+    if (X.plain && level + 1 != 16) sweep_batch_form<true>(P, S, X, level, tid, nthreads);
+    else sweep_batch_form<false>(P, S, X, level, tid, nthreads);
 }
 
 __device__ void book_batch_level(const TraversalParams& P, int level) {
@@ -1128,7 +1180,7 @@ bfs_batch_persistent(const __grid_constant__ TraversalParams P) {
             int level = 0;
             for (;; ++level) {
                 unsigned long long front_lanes = 0ull, pairs = 0ull;
-                if (threadIdx.x == 0) {   // in flight with the counters of the shape
+                if (threadIdx.x == 0 && P.full != nullptr) {   // in flight with the counters of the shape
                     front_lanes = ld_cg_u64(&P.ctl[level % 3].front_lanes);
                     pairs = ld_cg_u64(&P.ctl[level % 3].new_lanes);
                 }
@@ -1142,7 +1194,8 @@ bfs_batch_persistent(const __grid_constant__ TraversalParams P) {
                 const int dir = batch_direction(P, L, prev_bu);
                 if (dir == 2 && blockIdx.x == 0 && threadIdx.x == 0) P.stats->bu_levels += 1;
                 if (threadIdx.x == 0)
-                    open_sweep(P, s_sweep, front_lanes, pairs,
+                    open_sweep(P, s_sweep, front_lanes, pairs, L.cnt[0] + L.cnt[1] + L.cnt[2],
+                               L.edges[0] + L.edges[1] + L.edges[2],
                                L.edges[0] + L.edges[1] + L.edges[2] >= kManyEntries);
                 expand_level<true>(P, S, L, level, nullptr, dir);
                 prev_bu = dir == 2;
