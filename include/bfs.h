@@ -133,7 +133,9 @@ bfs_status bfs_graph_set_bins(bfs_graph* g, int32_t t_small, int32_t t_large,
  * paths; setting any of them switches to the kernel that does.  Results are
  * the same either way.  On a graph uploaded without BFS_UPLOAD_NO_RELABEL into
  * a context that allocates for itself, the default kernel also keeps 16 bytes
- * per vertex (row class counts) beside the graph when the device has room.
+ * per vertex (row class counts) beside the graph when 16 times as much is free
+ * at the upload (bfs_graph_info.device_bytes includes them); without them large
+ * levels read the entries that lead to visited vertices too.
  *   BFS_OPT_WARP_AGGREGATE   0/1: lanes of a warp that claim vertices in the
  *                            same 32-bit visited word merge their bits and
  *                            issue one atomicOr (default 0).
@@ -241,8 +243,10 @@ typedef struct bfs_run_stats {
     int64_t levels;         /* number of non-empty frontiers (max dist + 1) */
     int64_t reached;        /* vertices with dist >= 0 */
     int64_t edges_scanned;  /* m_c: sum of the out-degrees of the reached vertices --
-                               the entries a top-down traversal expands and the
-                               TEPS numerator in every direction mode */
+                               the entries of the rows a top-down traversal
+                               expands, also those it skips because they lead to
+                               visited vertices, and the TEPS numerator in every
+                               direction mode */
     int32_t status;         /* device-side status of the last traversal */
     int32_t bottom_up_levels; /* levels run bottom-up (BFS_OPT_DIRECTION) */
 } bfs_run_stats;
@@ -520,6 +524,13 @@ bfs_status bfs_debug_set_barrier_test(bfs_graph* g, int32_t stall, int64_t timeo
  * after its sweep -- for as many entries as fit; later entries are left
  * unwritten.  The timestamps cost one store per barrier. */
 bfs_status bfs_debug_set_timeline(bfs_graph* g, uint64_t* d_stamps, int32_t cap);
+
+/* For tests: levels of the default single-source traversal whose frontier has
+ * at least `entries` adjacency entries (>= 1; after the root's own level) mark
+ * and sweep instead of claiming and queueing, however small the graph; 0
+ * restores the default of 2^23.  Results are the same either way.  Must not be
+ * called while a traversal on g is in flight. */
+bfs_status bfs_debug_set_dense_min(bfs_graph* g, int64_t entries);
 
 #ifdef __cplusplus
 }

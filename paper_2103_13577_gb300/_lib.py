@@ -140,6 +140,7 @@ SIGNATURES = {
     "bfs_version": (_i32, []),
     "bfs_debug_set_barrier_test": (_i32, [_vp, _i32, _i64]),
     "bfs_debug_set_timeline": (_i32, [_vp, _vp, _i32]),
+    "bfs_debug_set_dense_min": (_i32, [_vp, _i64]),
     "bfs_run_static": (_i32, [_vp, _vp, _i64, _i64, _i32, _vp, _vp, _vp, ctypes.POINTER(RunStats)]),
     "bfs_run_paths": (_i32, [_vp, _vp, _vp, _vp, _i64, _i64, _i32, _i32, _i32, _vp, _vp, _vp,
                              ctypes.POINTER(PathsStats)]),

@@ -282,7 +282,7 @@ static void fill_params(bfs_graph* g, Workspace* ws, TraversalParams& P) {
     P.sweep_limit = sweep_limit(g);
     P.cut = g->d_cut;
     for (int c = 0; c < kCutClasses; ++c) P.cut_bound[c] = g->bounds.below[c];
-    P.dense_min = kDenseMin;
+    P.dense_min = g->dense_min;
     P.nnz = g->nnz;
     P.bu_limit = g->relabelled ? g->n_nonzero : g->n;
     P.dir_mode = g->dir_mode;
@@ -332,7 +332,7 @@ static bool plain_is_default(const bfs_graph* g) {
            g->use_match_any == 0 && g->l2_prefetch == 0;
 }
 static const void* default_plain_fn(const bfs_graph* g) {
-    return single_persistent_fn(g->min_blocks, may_run_dense(g->nnz, g->d_cut != nullptr));
+    return single_persistent_fn(g->min_blocks, may_run_dense(g->nnz, g->d_cut != nullptr, g->dense_min));
 }
 static const void* persistent_plain_fn(const bfs_graph* g) {
     return plain_is_default(g) ? default_plain_fn(g)
@@ -1114,6 +1114,15 @@ bfs_status bfs_debug_set_timeline(bfs_graph* g, uint64_t* d_stamps, int32_t cap)
     g->timeline = d_stamps;
     g->timeline_cap = d_stamps ? cap : 0;
     return BFS_OK;
+}
+
+bfs_status bfs_debug_set_dense_min(bfs_graph* g, int64_t entries) {
+    if (!g) return fail(BFS_ERR_INVALID_ARG, "null graph");
+    if (entries < 0) return fail(BFS_ERR_INVALID_ARG, "must be >= 0");
+    std::lock_guard<std::mutex> lk(g->mu);
+    cudaSetDevice(g->ctx->device);
+    g->dense_min = entries > 0 ? entries : kDenseMin;
+    return set_plain_grids(g);   // the other form of the kernel may have another grid
 }
 
 }  // extern "C"

@@ -94,8 +94,8 @@ constexpr long long kFilterMin = 1ll << 20;
 // sparse levels keep 64 registers with 112 / 148 bytes of spills and 14.2 KB of
 // shared memory per CTA where the form with both has 388 / 532 and 19.3 KB
 // (65 k vertices, 2.1 M entries: 96 us in the form with both, 77 without).
-inline bool may_run_dense(long long nnz, bool has_cut) {
-    return (has_cut ? 8 * nnz : nnz) >= kDenseMin;
+inline bool may_run_dense(long long nnz, bool has_cut, long long dense_min) {
+    return (has_cut ? 8 * nnz : nnz) >= dense_min;
 }
 
 struct TraversalParams {

@@ -92,6 +92,7 @@ struct bfs_graph {
     size_t graph_bytes = 0;
     int32_t grid_plain = 0, grid_batch = 0;
     int32_t debug_stall = 0;
+    long long dense_min = bfs::kDenseMin;   // tests lower it
     long long timeout_ns = 2000000000ll;
     int32_t use_match_any = 0;
     int32_t min_blocks = 4;           // resident CTAs per SM the kernels are built for
