@@ -132,18 +132,19 @@ __device__ __forceinline__ bool mbar_wait_bounded(const TraversalParams& P,
 // ------------------------------------------------------------ grid barrier
 // All CTAs are co-resident (cooperative launch).  Thread 0 of each CTA adds
 // its arrival to one 64-bit word that only grows during a launch: the k-th
-// barrier is complete once the word reaches k * gridDim.x, so an arrival is
-// a fire-and-forget reduction and the wait is a loop of acquire loads (no
-// reset or generation step that the last arrival would have to publish with
-// further round trips).  An acquire load throws away the SM's L1: where some
-// CTAs of an SM wait long while others still expand (long_wait, the dense
-// levels), the loop polls with relaxed loads and fences once at its end
-// (scale 22, level 2: 222 -> 196 us; on short waits the fence costs 0.3 us).  Bit 63 of the word says that a CTA gave up: a wait
-// longer than timeout_ns of %globaltimer records kDevTimeout, sets the bit
-// and returns false, and every CTA that reads the bit returns false too.
-// `epoch` (thread 0's, in shared memory: no register held across the level
-// loop) counts the barriers this CTA has passed in the launch, the same in
-// every CTA; the last CTA to leave the launch clears the word.
+// barrier is complete once the word reaches k * gridDim.x, so an arrival is a
+// fire-and-forget reduction and the wait is a loop of acquire loads (no reset
+// or generation step that the last arrival would have to publish with further
+// round trips).  An acquire load throws away the SM's L1: where some CTAs of
+// an SM wait long while others still expand (long_wait, the dense levels), the
+// loop polls with relaxed loads and fences once at its end (scale 22, level 2:
+// 222 -> 196 us; on short waits the fence costs 0.3 us).  Bit 63 of the word
+// says that a CTA gave up: a wait longer than timeout_ns of %globaltimer
+// records kDevTimeout, sets the bit and returns false, and every CTA that
+// reads the bit returns false too. `epoch` (thread 0's, in shared memory: no
+// register held across the level loop) counts the barriers this CTA has passed
+// in the launch, the same in every CTA; the last CTA to leave the launch
+// clears the word.
 constexpr unsigned long long kBarGaveUp = 1ull << 63;
 
 __device__ __forceinline__ unsigned long long ld_acquire_u64(const unsigned long long* p) {
@@ -593,8 +594,8 @@ __device__ __forceinline__ void visit_plain_k(const TraversalParams& P, Stage<fa
 // not seen yet into next[u].  visited only changes in phase B, so a cached
 // value is a safe filter; next[u] is read first so that lanes already
 // present skip the atomic (a fire-and-forget red.or otherwise).
-// The K pairs are read in groups of kBatchProbeGroup (4 at 3 CTAs/SM: 8
-// would keep 32 registers of pairs live, which spills at that occupancy).
+// The K pairs are read in groups of 4 (8 would keep 32 registers of pairs
+// live, which spills at 3 CTAs per SM).
 // Once many vertices have been reached by every live lane, their bitmap
 // (n / 8 bytes, mostly L1 hits in degree order) is read first: it spares two
 // thirds of a scale-20 launch's level 3 entries and nearly all of level 4's

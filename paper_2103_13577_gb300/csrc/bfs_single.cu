@@ -260,15 +260,18 @@ __device__ __forceinline__ void open_level(const TraversalParams& P, Level& L, i
                         __shfl_sync(FULL_MASK, cnt, 2);
     const int fit = (63 - __clzll(E1 + E2 + 1)) - (31 - __clz(gridDim.x * kWarps));
     const unsigned long long reached = L.reached + discovered;
-    // Dense pays from 8 M entries on; from 1 M on where the targets are spread
-    // (no hubs) or a quarter of the vertices is reached, so that most entries
-    // lead nowhere new.  Below that, and on a skewed graph's early levels, the
-    // marks crowd into the few bitmap lines of the hubs (a reduction takes
-    // ~2.3 ns of its 128-byte line's time) and the extra barrier and sweep
-    // are not won back: 200 k vertices, 4.5 M entries: sparse 42 us, dense 56;
-    // a million vertices, 6.1 M entries: 70 and 75; 18 M: 89 and 88; scale
-    // 22, 67 M: 190 and 180.  With most vertices reached 13 M entries take 50
-    // and 37 us; uniform, 20 M entries: 121 and 100.
+    // Dense pays from 8 M entries on; from 1 M on where the targets are spread (no
+    // hubs) or a quarter of the vertices is reached, so that most entries lead
+    // nowhere new, and the rows' class counts are kept, so that they skip them.
+    // (Without the counts, as in a caller's arena, the lower limit took the skewed
+    // graph of 262 k vertices from 108 to 120 us and a uniform one of a million
+    // from 261 to 240: left out.)  Below that, and on a skewed graph's early
+    // levels, the marks crowd into the few bitmap lines of the hubs (a reduction
+    // takes ~2.3 ns of its 128-byte line's time) and the extra barrier and sweep
+    // are not won back: 200 k vertices, 4.5 M entries: sparse 42 us, dense 56; a
+    // million vertices, 6.1 M entries: 70 and 75; 18 M: 89 and 88; scale 22, 67 M:
+    // 190 and 180.  With most vertices reached 13 M entries take 50 and 37 us;
+    // uniform, 20 M entries: 121 and 100.
     const bool hubs = P.cut != nullptr && P.cut_bound[kHubClass] > 0;
     const bool late = 4 * (long long)reached > P.sweep_limit;
     const bool dense = kDense && (E >= P.dense_min ||
@@ -662,15 +665,15 @@ struct SweepShared {
     QueueShared queue;
 };
 
-// After a dense level: every vertex whose visited bit was set during the
-// level (it is not in `queued` yet) gets distance level + 1 and a place in
-// the next frontier.  A CTA takes 64 bitmap words at a time, spread evenly
-// over the bitmap: in degree order the heavy vertices, whose chunk-start
-// runs are the longest, would otherwise all fall to a few CTAs (sweep of a
-// scale-22 traversal's level 2: 49 us with consecutive words, 40 spread).  A word's 32 row
-// offsets and caller numbers are read in order.  The first word with a
-// vertex still unvisited bounds the prefix of the order that the next
-// level's rows may skip.
+// After a dense level: every vertex whose visited bit was set during the level
+// (it is not in `queued` yet) gets distance level + 1 and a place in the next
+// frontier.  A CTA takes 64 bitmap words at a time, spread evenly over the
+// bitmap: in degree order the heavy vertices, whose chunk-start runs are the
+// longest, would otherwise all fall to a few CTAs (sweep of a scale-22
+// traversal's level 2: 49 us with consecutive words, 40 spread).  A word's 32
+// row offsets and caller numbers are read in order.  The first word with a
+// vertex still unvisited bounds the prefix of the order that the next level's
+// rows may skip.
 __device__ void sweep_level(const TraversalParams& P, SweepShared& X, int level) {
     const unsigned lane = lane_id();
     const int warp = threadIdx.x >> 5;
