@@ -43,11 +43,20 @@ import numpy as np  # noqa: E402
 SCALE, EDGE_FACTOR, GRAPH_SEED, ROOT_SEED, NROOTS = 22, 16, 22, 3, 64
 METRIC = "BFS GTEPS (hmean over 64 roots) plain vs 64-root batched; query p50/p99 latency"
 WORKLOAD = "kronecker_s22_ef16_plain_64roots"
-KERNEL_SRC = os.path.join(ROOT, "paper_2103_13577_gb300", "csrc", "bfs_kernels.cu")
-TRAFFIC_FILE = os.path.join(ROOT, "profiles", "bfs_plain_persistent_kron_s22_traffic.json")
+CSRC = os.path.join(ROOT, "paper_2103_13577_gb300", "csrc")
+KERNEL_SRC = os.path.join(CSRC, "bfs_single.cu")
+# the single-source and the batched kernel and what both are built from: a
+# traffic record of either holds while none of them changes
+TRAVERSAL_SRCS = [KERNEL_SRC] + [os.path.join(CSRC, f) for f in
+                                 ("bfs_kernels.cu", "bfs_device.cuh", "bfs_internal.h")]
+TRAFFIC_FILE = os.path.join(ROOT, "profiles", "bfs_single_persistent_kron_s22_traffic.json")
 BATCH_TRAFFIC_FILE = os.path.join(ROOT, "profiles", "bfs_batch_persistent_kron_s22_traffic.json")
-PATHS_SRC = os.path.join(ROOT, "paper_2103_13577_gb300", "csrc", "bfs_paths.cu")
+PATHS_SRC = os.path.join(CSRC, "bfs_paths.cu")
 PATHS_TRAFFIC_FILE = os.path.join(ROOT, "profiles", "paths_persistent_kron_s22_traffic.json")
+
+
+NOMINAL = ("nominal work: every column entry of the expanded rows once, also those the kernel "
+           "skips because they lead to visited vertices; traffic is what it moves (ncu)")
 
 
 def env_int(name, default):
@@ -78,8 +87,11 @@ def measured_hbm_peak():
 
 
 def kernel_hash(src=KERNEL_SRC):
-    with open(src, "rb") as f:
-        return hashlib.sha256(f.read()).hexdigest()[:16]
+    h = hashlib.sha256()
+    for path in TRAVERSAL_SRCS if src in TRAVERSAL_SRCS else [src]:
+        with open(path, "rb") as f:
+            h.update(f.read())
+    return h.hexdigest()[:16]
 
 
 def recorded_traffic(path=TRAFFIC_FILE, src=KERNEL_SRC):
@@ -186,7 +198,7 @@ def batch_frontier_sums(rows, deg):
 
 
 def batch_algorithmic_bytes(sizes, degs, reached: int, n: int, k: int, elem: int) -> float:
-    """Bytes one top-down batched launch (bfs_batch_persistent) has to move,
+    """Nominal bytes of one top-down batched launch (bfs_batch_persistent),
     each item once:
       init      16 N                 visited/next lane-set pairs cleared
       level L   4 D_L                column entries of the frontier's rows
@@ -198,7 +210,10 @@ def batch_algorithmic_bytes(sizes, degs, reached: int, n: int, k: int, elem: int
                                      level rows of the reached ones
                 + k N elem           the k distance rows
     Lane-set updates of the neighbours (atomicOr on next) and the level-row
-    re-reads of vertices reached before are cache traffic, not counted."""
+    re-reads of vertices reached before are cache traffic, not counted.  A
+    measure of the work, the same for every kernel, and not of what this one
+    moves: rows skip the entries that lead to vertices every lane has, and
+    levels below 16 touch 32 of a level row's 64 bytes."""
     per_level = sum(4 * d + 120 * a + 16 * n for a, d in zip(sizes, degs))
     return float(per_level + 16 * n + 12 * n + 64 * reached + k * n * elem)
 
@@ -499,7 +514,7 @@ def gpu_arm(args, rank, world, local_rank):
     g.set_option(bfs.BFS_OPT_DIRECTION, 0)
     batch_do_ms = bev[0].elapsed_time(bev[1]) / reps
 
-    # roofline of the traversal kernel (one launch per root)
+    # roofline of the traversal kernel (one launch per root), on nominal work
     peak, peak_kind = measured_hbm_peak()
     b_achieved = b_bytes / (batch_ms * 1e-3) / 1e9
     alg_bytes = 4.0 * m_c + 32.0 * n_c + 8.125 * n
@@ -540,7 +555,7 @@ def gpu_arm(args, rank, world, local_rank):
                     "d2h_bytes_per_step": 2 * 4 * n * NROOTS},
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                          "frac": achieved / peak, "traffic": traffic,
-                         "kernel": "bfs_plain_persistent",
+                         "kernel": "bfs_single_persistent", "bytes": NOMINAL,
                          "peak_source": f"{peak_kind} (MEASURED_PEAKS.json hbm_gbs)"
                          if peak_kind == "measured" else "fallback 6.8 TB/s",
                          "algorithmic_bytes_per_launch": float(alg_bytes.mean())},
@@ -561,7 +576,7 @@ def gpu_arm(args, rank, world, local_rank):
                         "roofline": {"bound": "hbm", "achieved": b_achieved, "peak": peak,
                                      "unit": "GB/s", "frac": b_achieved / peak,
                                      "traffic": recorded_traffic(BATCH_TRAFFIC_FILE),
-                                     "kernel": "bfs_batch_persistent",
+                                     "kernel": "bfs_batch_persistent", "bytes": NOMINAL,
                                      "algorithmic_bytes_per_launch": b_bytes,
                                      "frontier_entries": int(sum(b_sizes)),
                                      "frontier_edges": int(sum(b_degs))},

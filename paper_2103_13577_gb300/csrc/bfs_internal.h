@@ -84,8 +84,8 @@ constexpr long long kDenseMin = 1ll << 23;
 // Entries from which a batched top-down run looks for vertices that every live
 // lane has reached.  A graph of fewer gives a warp a few hundred entries per
 // level at most, and the counters cost its levels more than the entries spared
-// (64 lanes, 50 k vertices, 0.8 M entries: 154 us with them, 146 without; 131 k,
-// 2 M: 186 either way, and 600 k, 9 M: 386 with them against 411).
+// (64 lanes, 50 k vertices, 0.8 M entries: 151 us with them, 147 without; 131 k,
+// 2 M: 190 either way; 600 k, 9 M: 386 with them, 412 before there were any).
 constexpr long long kFilterMin = 1ll << 20;
 
 // Whether a level of a graph of nnz entries can run dense (a level never holds

@@ -11,8 +11,9 @@
 //    parent stored -- and, after a grid barrier, a sweep over the bitmap
 //    writes the distances of the vertices marked since the previous level
 //    and queues them.
-// Runs that ask for direction-optimizing levels, bitmap-order levels or one
-// of the tuning options use bfs_kernels.cu.
+// The kernel has a form without dense levels for graphs that cannot have one
+// (may_run_dense) and for bfs_run_static.  Runs that ask for direction-optimizing
+// levels, bitmap-order levels or one of the tuning options use bfs_kernels.cu.
 #define BFS_LEAN_PATHS 1
 #include "bfs_device.cuh"
 
