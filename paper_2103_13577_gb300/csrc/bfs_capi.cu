@@ -30,7 +30,7 @@ cudaError_t launch_degree_bins(const int64_t* off, long long n, int t_small, int
 size_t relabel_scratch_bytes(long long n);
 cudaError_t relabel_graph(const int64_t* off, const int32_t* col, long long n, long long nnz,
                           int sms, int32_t* new2old, int32_t* old2new, int64_t* new_off,
-                          int32_t* new_col, void* scratch, uint16_t* cut, CutBounds* bounds,
+                          int32_t* new_col, void* scratch, bool keep_cut, CutBounds* bounds,
                           cudaStream_t s);
 
 static thread_local std::string t_last_error;
@@ -820,20 +820,25 @@ bfs_status bfs_graph_upload(bfs_context* ctx, const int64_t* row_off, const int3
             return cleanup(fail(BFS_ERR_NO_MEMORY, "device memory exhausted (renumbering)"));
         }
         // The rows' class counts (16 bytes per vertex) are an addition that a
-        // traversal can do without: they are kept only where the library
-        // allocates for itself (a caller's arena keeps the sizes it always
-        // had) and the device has ample room for what comes after them.
-        const size_t cut_bytes = (size_t)n * kCutClasses * sizeof(uint16_t);
+        // traversal can do without: they are kept, in the renumbering's
+        // scratch, only where the library allocates for itself (a caller's
+        // arena keeps the sizes it always had) and the device has ample room
+        // for what comes after them.
+        const size_t cut_bytes = round_up(relabel_scratch_bytes(n), kAlign);
         size_t mem_free = 0, mem_all = 0;
-        if (m->capacity() == 0 && cudaMemGetInfo(&mem_free, &mem_all) == cudaSuccess &&
-            mem_free / 16 > cut_bytes)
-            g->d_cut = static_cast<uint16_t*>(m->alloc(cut_bytes));
-        if (g->d_cut) g->graph_bytes += round_up(cut_bytes, kAlign);
+        const bool keep_cut = m->capacity() == 0 &&
+                              cudaMemGetInfo(&mem_free, &mem_all) == cudaSuccess &&
+                              mem_free / 16 > cut_bytes;
         e = relabel_graph(g->d_off, g->d_col, n, nnz, ctx->sms, g->d_new2old, g->d_old2new, n_off,
-                          n_col, scratch, g->d_cut, &g->bounds, s);
+                          n_col, scratch, keep_cut, &g->bounds, s);
         if (e == cudaSuccess) e = cudaMemsetAsync(n_col + nnz, 0, 16 * 4, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-        m->release(scratch);
+        if (e == cudaSuccess && keep_cut) {
+            g->d_cut = static_cast<uint16_t*>(scratch);
+            g->graph_bytes += cut_bytes;
+        } else {
+            m->release(scratch);
+        }
         if (e != cudaSuccess) {
             m->release(n_off);
             m->release(n_col);

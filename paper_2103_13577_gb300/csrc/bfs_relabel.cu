@@ -124,7 +124,7 @@ __global__ void rel_bounds_kernel(const unsigned long long* key_start, long long
 // warp: 128 entries are read together, and the 9 classes of a chunk are told
 // apart by the ballots of their number's 4 bits (a ballot per class and one
 // chunk at a time: upload of scale 22, 16 edges per vertex, 13.3 ms, of a star
-// of 2 M vertices 113; now 8.5 and 52).
+// of 2 M vertices 113; now 8.3 and 49).
 constexpr int kStep = 4;   // 32-entry chunks of a row in flight
 __device__ __forceinline__ void read_entries(const int32_t* old2new, const int32_t* row, unsigned d,
                                              unsigned k, int32_t (&x)[kStep]) {
@@ -306,7 +306,8 @@ cudaError_t exclusive_scan_i64(const int64_t* in, long long n, int64_t* out, int
     return cudaMemcpyAsync(out + n, tmp + nb, sizeof(int64_t), cudaMemcpyDeviceToDevice, s);
 }
 
-// Scratch sizes (bytes) the relabel needs beyond the new graph arrays.
+// Scratch sizes (bytes) the relabel needs beyond the new graph arrays; the
+// first 16 n of them hold the rows' class counts when those are kept.
 size_t relabel_scratch_bytes(long long n) {
     const long long ntiles = (n + kRelTile - 1) / kRelTile;
     const long long table = (long long)kBuckets * ntiles;
@@ -314,13 +315,16 @@ size_t relabel_scratch_bytes(long long n) {
     return (size_t)(2 * (big + 1) * 8 + ((big + kScanBlock - 1) / kScanBlock + 2) * 8) + 1024;
 }
 
-// Builds new2old/old2new and the renumbered CSR (new_off[n+1], new_col[nnz]);
-// cut (nullable, [kCutClasses][n]) and bounds (host, written when the stream
-// has been waited for) describe the rows' degree classes.
+// Builds new2old/old2new and the renumbered CSR (new_off[n+1], new_col[nnz]).
+// With keep_cut the rows' class counts, uint16[kCutClasses][n], are left at
+// the start of scratch, which the caller then keeps; bounds (host) are written
+// when the stream has been waited for.
 cudaError_t relabel_graph(const int64_t* off, const int32_t* col, long long n, long long nnz,
                           int sms, int32_t* new2old, int32_t* old2new, int64_t* new_off,
-                          int32_t* new_col, void* scratch, uint16_t* cut, CutBounds* bounds,
+                          int32_t* new_col, void* scratch, bool keep_cut, CutBounds* bounds,
                           cudaStream_t s) {
+    static_assert(kCutClasses * sizeof(uint16_t) <= 2 * sizeof(int64_t), "the counts fit in a and b");
+    static_assert(sizeof(CutBounds) <= 1024, "the bounds fit in tmp");
     const long long ntiles = (n + kRelTile - 1) / kRelTile;
     const long long table = (long long)kBuckets * ntiles;
     const long long big = table > n ? table : n;
@@ -336,8 +340,10 @@ cudaError_t relabel_graph(const int64_t* off, const int32_t* col, long long n, l
     rel_newdeg_kernel<<<sms * 4, 256, 0, s>>>(off, new2old, n, a);
     e = exclusive_scan_i64(a, n, new_off, tmp, s);
     if (e != cudaSuccess) return e;
-    // the scan's scratch is free again: the class bounds go there
-    CutBounds* d_bounds = reinterpret_cast<CutBounds*>(a);
+    // the scan's scratch is free again: the class bounds go there; after them
+    // a and b are free too, for the class counts
+    CutBounds* d_bounds = reinterpret_cast<CutBounds*>(tmp);
+    uint16_t* cut = keep_cut ? static_cast<uint16_t*>(scratch) : nullptr;
     rel_bounds_kernel<<<1, 32, 0, s>>>(reinterpret_cast<const unsigned long long*>(b), ntiles, d_bounds);
     rel_columns_kernel<<<sms * 8, 256, 0, s>>>(off, col, new2old, old2new, new_off, n, d_bounds, cut,
                                                 new_col);
