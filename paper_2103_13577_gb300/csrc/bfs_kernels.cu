@@ -989,8 +989,11 @@ __device__ void sweep_batch_form(const TraversalParams& P, Stage<true>& S, Sweep
     const uint64_t all_lanes = lanes_of(P);
     // kSweepUnroll vertices per thread and pass, their lane-set pairs loaded
     // together; the trip count is the same for every thread (the stage push
-    // is warp-collective)
-    constexpr int kSweepUnroll = 4;
+    // is warp-collective).  Two in the plain form: half the code of four, and
+    // enough for the few vertices that its graphs have per thread (64 lanes, 65 k
+    // vertices with a path of 300: 3373 -> 3274 us; one: 5 lanes on a 300 x 300
+    // mesh 7107 -> 7457).
+    constexpr int kSweepUnroll = kPlain ? 2 : 4;
     const long long stride = nthreads * kSweepUnroll;
     const long long nround = (P.n + stride - 1) / stride * stride;
     ulonglong2* const pairs = reinterpret_cast<ulonglong2*>(P.lane_vn);
